@@ -282,8 +282,10 @@ def prepare(case, seed):
     elif kind == "batch":
         sizes = _sizes(case, seed)
         A = [_csr_tuple(*_sparse_csr(n, case["inside"], 100 * seed + p)[:3]) for p, n in enumerate(sizes)]
+        # the shifted systems two digits below the eigenpairs' tolerance, so that the outer iteration ends by
+        # converging and not at the noise of its inner solves
         st["ctx"] = F.FeastBatch(A, [_sparse_contour(case["ne"])] * len(A), case["m0"], precision=F.PREC_FP32_IR,
-                                 inner_max=8, max_iter=30)
+                                 inner_tol=1e-12, inner_max=8, max_iter=30)
         st["Y"], st["Yh"] = _start(sum(sizes), case["m0"], seed)
         st["ref"] = [_normal(17, n).to(torch.complex128) for n in sizes]
     else:
