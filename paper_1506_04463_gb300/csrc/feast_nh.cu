@@ -106,7 +106,7 @@ struct feast_nh_ctx {
   void *Rn = nullptr, *Rhn = nullptr;
   double *part = nullptr;
   double *bynorm2 = nullptr;
-  int *d_done = nullptr, *d_err = nullptr, *d_ext = nullptr;
+  int *d_err = nullptr, *d_ext = nullptr;
   int *d_fxy = nullptr;  // column exponent fields of the tensor-core projections
   double *d_maxrel = nullptr;
   cxd *BQ = nullptr, *gam = nullptr, *V = nullptr, *Vinv = nullptr, *S = nullptr, *Sh = nullptr, *AU = nullptr,
@@ -398,7 +398,6 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
       }
       launch_cxf_accumulate(X, ctx->dfg, (size_t)ne * n * m, mode, ctx->s);
     };
-    CKC(cudaMemsetAsync(ctx->d_done, 0, sizeof(int), ctx->s));
     launch_broadcast_cxf(BY, (cxf *)ctx->Rn, (size_t)n * m, ne, ctx->s);
     fg(0, (const cxf *)ctx->Rn, ctx->Xn, 0);
     if (!cs) {
@@ -423,14 +422,11 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
                                           nullptr, ctx->part + (size_t)gm * ne * m, m, nullptr, ctx->s);
         ev_end(ctx, ctx->ev_resid, kr);
       }
-      launch_residual_check(ctx->part, gm, ne, m, ctx->bynorm2, cs ? 1 : 2, inner_tol, ctx->d_maxrel, ctx->d_done,
-                            ctx->s);
-      CKC(cudaMemcpyAsync(ctx->h_small + 2, ctx->d_done, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+      launch_residual_check(ctx->part, gm, ne, m, ctx->bynorm2, cs ? 1 : 2, ctx->d_maxrel, ctx->s);
+      CKC(cudaMemcpyAsync(ctx->h_small, ctx->d_maxrel, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
       CKC(cudaStreamSynchronize(ctx->s));
-      int done = 0;
-      std::memcpy(&done, ctx->h_small + 2, sizeof(int));
       ctx->inner_steps = it + 1;
-      if (done) break;
+      if (ctx->h_small[0] <= inner_tol) break;
       if (it + 1 < steps) {
         fg(0, (const cxf *)ctx->Rn, ctx->Xn, 1);
         if (!cs) fg(1, (const cxf *)ctx->Rhn, ctx->Xhn, 1);
@@ -443,7 +439,6 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
     // form) or FP64 factors (plain form; the unpivoted factors of a general
     // pencil can lose accuracy, which the refinement restores or reports)
     const bool f32 = fp32(ctx);
-    CKC(cudaMemsetAsync(ctx->d_done, 0, sizeof(int), ctx->s));
     auto solve = [&](const void *rR, const void *rL, size_t rns, int mode) {
       const int k = ev_begin(ctx, ctx->ev_solve);
       if (f32)
@@ -503,15 +498,12 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
                                              nullptr, pl, m, nullptr, ctx->s);
         ev_end(ctx, ctx->ev_resid, kr);
       }
-      launch_residual_check(ctx->part, gm, ne, m, ctx->bynorm2, cs ? 1 : 2, inner_tol, ctx->d_maxrel, ctx->d_done,
-                            ctx->s);
-      // one 4-byte read per refinement step decides whether to go on
-      CKC(cudaMemcpyAsync(ctx->h_small + 2, ctx->d_done, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+      launch_residual_check(ctx->part, gm, ne, m, ctx->bynorm2, cs ? 1 : 2, ctx->d_maxrel, ctx->s);
+      // one 8-byte read per refinement step decides whether to go on
+      CKC(cudaMemcpyAsync(ctx->h_small, ctx->d_maxrel, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
       CKC(cudaStreamSynchronize(ctx->s));
-      int done = 0;
-      std::memcpy(&done, ctx->h_small + 2, sizeof(int));
       ctx->inner_steps = it + 1;
-      if (done) break;
+      if (ctx->h_small[0] <= inner_tol) break;
       if (it + 1 < steps) solve(ctx->Rn, cs ? nullptr : ctx->Rhn, xns, 1);
     }
     launch_node_sum(ne, ctx->dw, ctx->Xn, xns, n, m, Q, ctx->s);
@@ -962,7 +954,6 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     ctx->gmax = spmm_max_grid();
     ctx->part = dalloc<double>(ctx, inner ? (size_t)2 * ctx->gmax * 2048 * sizeof(double) : 16);
     ctx->bynorm2 = dalloc<double>(ctx, 2 * kMaxM0 * sizeof(double));
-    ctx->d_done = dalloc<int>(ctx, sizeof(int));
     ctx->d_err = dalloc<int>(ctx, sizeof(int));
     ctx->d_maxrel = dalloc<double>(ctx, sizeof(double));
     ctx->d_piv = dalloc<double>(ctx, 2 * sizeof(double));

@@ -11,9 +11,11 @@
 // twice (one pass for the dot products of all previous basis vectors, one
 // for the update, repeated).  Scalars and the small least-squares problems
 // are FP64.  Converged systems are frozen (their columns are skipped).
+#include <algorithm>
 #include <vector>
 
 #include "kernels.h"
+#include "reduce.cuh"
 
 namespace {
 constexpr int kFgMaxK = 64;
@@ -37,13 +39,20 @@ __global__ void __launch_bounds__(kFgThreads) k_fg_dots(const cxf *const *V, int
     }
   }
 }
-// out[l][s] = sum_chunks partial (fixed order); also optionally |w|^2 sums
-__global__ void k_fg_dots_reduce(const cxd *partial, int nchunks, int nv, int S, cxd *out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nv * S) return;
-  cxd acc = mk(0.0, 0.0);
-  for (int p = 0; p < nchunks; ++p) acc = acc + partial[(size_t)p * nv * S + e];
-  out[e] = acc;
+// out[l][s] = sum over the chunks of partial (fixed order): one CTA per 2
+// outputs, 128 threads each.  A thread per output took 167 us at 1000 chunks
+// (three quarters of an FGMRES solve).
+constexpr int kFdC = 2, kFdR = 128;
+__global__ void __launch_bounds__(kFdC *kFdR) k_fg_dots_reduce(const cxd *__restrict__ partial, int nchunks, int count,
+                                                               cxd *out) {
+  __shared__ cxd sm[kFdC * kFdR];
+  const int e = blockIdx.x * kFdC + threadIdx.x % kFdC;
+  const cxd s = column_sum<kFdC, kFdR>(partial, nchunks, count, e, e < count, sm);
+  if (e < count && threadIdx.x < kFdC) out[e] = s;
+}
+static void fg_dots_reduce(const cxd *partial, int nchunks, int count, cxd *out, cudaStream_t s) {
+  k_fg_dots_reduce<<<ceil_div(count, kFdC), kFdC * kFdR, 0, s>>>(partial, nchunks, count, out);
+  note_launch();
 }
 // w -= sum_l h[l][s] V_l ; H[s][l][col] += h[l][s] (the Gram-Schmidt coefficients)
 __global__ void k_fg_orth_update(const cxf *const *V, int nv, const cxd *h, cxf *w, int ne, int n, int m,
@@ -182,17 +191,18 @@ __global__ void k_fg_sub(const cxf *b, const cxf *o, cxf *r, size_t count) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
     r[e] = b[e] - o[e];
 }
-// Jacobi / identity preconditioner: z = v / (z_j b_ii - a_ii) (diag given) or z = v
-__global__ void k_fg_jacobi(const cxf *v, const cxd *zn, int conj_z, const cxd *adiag, const cxd *bdiag, cxf *z,
-                            int ne, int n, int m) {
-  const size_t count = (size_t)ne * n * m;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t j = e / ((size_t)n * m), rem = e - j * n * m;
-    const int i = (int)(rem / m);
-    if (!adiag) {
-      z[e] = v[e];
-      continue;
-    }
+// Jacobi preconditioner: z = v / (z_j b_ii - a_ii).  The FP64 quotient of a
+// (node, row) serves its m columns: a CTA forms the quotients of 256 rows of
+// one node, a row a thread, and then streams the rows' m columns.  With the
+// quotient formed by every element the kernel was bound by the FP64 pipe
+// (49 us for 768k elements, of which the data takes 2).
+__global__ void __launch_bounds__(256) k_fg_jacobi(const cxf *__restrict__ v, const cxd *__restrict__ zn, int conj_z,
+                                                   const cxd *__restrict__ adiag, const cxd *__restrict__ bdiag,
+                                                   cxf *__restrict__ z, int n, int m, int rows) {
+  __shared__ cxf inv[256];
+  const int j = blockIdx.y, i0 = blockIdx.x * rows, cnt = min(rows, n - i0);
+  if ((int)threadIdx.x < cnt) {
+    const int i = i0 + threadIdx.x;
     cxd zj = zn[j];
     if (conj_z) zj = conj(zj);
     cxd a = adiag[i], bd = bdiag ? bdiag[i] : mk(1.0, 0.0);
@@ -200,9 +210,11 @@ __global__ void k_fg_jacobi(const cxf *v, const cxd *zn, int conj_z, const cxd *
       a = conj(a);
       bd = conj(bd);
     }
-    const cxd dd = zj * bd - a;
-    z[e] = ccast<float>(cdiv(mk(1.0, 0.0), dd)) * v[e];
+    inv[threadIdx.x] = ccast<float>(cdiv(mk(1.0, 0.0), zj * bd - a));
   }
+  __syncthreads();
+  const size_t base = ((size_t)j * n + i0) * m;
+  for (int e = threadIdx.x; e < cnt * m; e += 256) z[base + e] = inv[e / m] * v[base + e];
 }
 
 // ---------------------------------------------------------------------------
@@ -271,8 +283,7 @@ void fg_dots(FgWork &f, int nv, const cxf *w, int ne, int n, int m, cudaStream_t
   chunks = ceil_div(n, rpc);
   k_fg_dots<<<chunks, kFgThreads, 0, s>>>(f.dV, nv, w, ne, n, m, rpc, f.sc.active, f.partial);
   note_launch();
-  k_fg_dots_reduce<<<ceil_div(nv * S, 256), 256, 0, s>>>(f.partial, chunks, nv, S, f.dots);
-  note_launch();
+  fg_dots_reduce(f.partial, chunks, nv * S, f.dots, s);
 }
 }  // namespace
 
@@ -346,8 +357,7 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
         const int rpc = ceil_div(n, chunks);
         k_fg_dots<<<chunks, kFgThreads, 0, s>>>(dv, 1, f.w, ne, n, m, rpc, f.sc.active, f.partial);
         note_launch();
-        k_fg_dots_reduce<<<ceil_div(S, 256), 256, 0, s>>>(f.partial, chunks, 1, S, f.dots);
-        note_launch();
+        fg_dots_reduce(f.partial, chunks, S, f.dots, s);
       }
       cudaMemcpyAsync(f.dV + kmax, &hv[kmax], sizeof(void *), cudaMemcpyHostToDevice, s);
       cudaMemsetAsync(f.sc.nact, 0, sizeof(int), s);
@@ -400,7 +410,9 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
 
 void launch_fg_jacobi(const cxf *v, const cxd *zn, int conj_z, const cxd *adiag, const cxd *bdiag, cxf *z, int ne,
                       int n, int m, cudaStream_t s) {
-  k_fg_jacobi<<<grid_for((size_t)ne * n * m), 256, 0, s>>>(v, zn, conj_z, adiag, bdiag, z, ne, n, m);
+  // enough CTAs for the chip first, then up to 256 rows of a quotient each
+  const int rows = std::max(1, (int)std::min<long long>(256, ((long long)n * ne + 607) / 608));
+  k_fg_jacobi<<<dim3(ceil_div(n, rows), ne), 256, 0, s>>>(v, zn, conj_z, adiag, bdiag, z, n, m, rows);
   note_launch();
 }
 

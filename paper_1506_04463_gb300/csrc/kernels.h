@@ -59,11 +59,11 @@ template <typename Tout>
 int launch_multishift_residual_capped(const CsrView &A, const CsrView *B, int ne, const cxd *d_z, const cxd *d_w,
                                       const cxd *X, const cxd *BY, cx<Tout> *R, cxd *Q, double *partial, int m,
                                       int max_grid, cudaStream_t s);
-// Reduce the partial sums into relative residuals ||R_jc|| / ||BY_c|| and set
-// *d_done = 1 when all are <= tol.  bynorm2[c] = ||BY_c||^2.  nsides blocks of
-// partials (each nparts x ne*m) and of bynorm2 (each m) are checked together.
+// *d_maxrel = the largest relative residual ||R_jc|| / ||BY_c|| (infinity if one
+// is NaN).  bynorm2[c] = ||BY_c||^2.  nsides blocks of partials (each nparts x
+// ne*m) and of bynorm2 (each m) are checked together.
 void launch_residual_check(const double *partial, int nparts, int ne, int m, const double *bynorm2, int nsides,
-                           double tol, double *d_maxrel, int *d_done, cudaStream_t s);
+                           double *d_maxrel, cudaStream_t s);
 // FP32 multi-shift operator V_j = (z_j B - A) P_j (conj_z: conj(z_j), for the
 // conjugate-transpose CSR pair) over node-major complex-float blocks; returns
 // the grid used.  grid_per_sm <= 0: 8 CTAs of 256 threads per SM.

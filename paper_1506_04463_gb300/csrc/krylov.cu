@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "reduce.cuh"
 
 namespace {
 constexpr int kDotThreads = 256;
@@ -56,14 +57,14 @@ __global__ void __launch_bounds__(kDotThreads) k_coldots(DotArgs d, int n, int P
   }
 }
 
-// Sum the partials (fixed order) into out[k][pair].
-__global__ void k_dots_reduce(const cxd *part, int nparts, int P, int nd, cxd *out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nd * P) return;
-  const int k = e / P, pair = e - k * P;
-  cxd s = mk(0.0, 0.0);
-  for (int p = 0; p < nparts; ++p) s = s + part[((size_t)k * nparts + p) * P + pair];
-  out[e] = s;
+// Sum the partials (fixed order) into out[k][pair]: dot k = blockIdx.y, one
+// CTA per 2 pairs with 128 threads each.
+constexpr int kDrC = 2, kDrR = 128;
+__global__ void __launch_bounds__(kDrC *kDrR) k_dots_reduce(const cxd *__restrict__ part, int nparts, int P, cxd *out) {
+  __shared__ cxd sm[kDrC * kDrR];
+  const int pair = blockIdx.x * kDrC + threadIdx.x % kDrC, k = blockIdx.y;
+  const cxd s = column_sum<kDrC, kDrR>(part + (size_t)k * nparts * P, nparts, P, pair, pair < P, sm);
+  if (pair < P && threadIdx.x < kDrC) out[(size_t)k * P + pair] = s;
 }
 
 // Scalar updates.  Notation: the operator output holds V' = -M P, T' = -M S.
@@ -210,7 +211,7 @@ static void coldots(const DotArgs &d, int n, int P, int m, size_t xns, cxd *part
   const int rpc = ceil_div(n, g0), g = ceil_div(n, rpc);
   k_coldots<<<g, kDotThreads, 0, s>>>(d, n, P, m, xns, rpc, part);
   note_launch();
-  k_dots_reduce<<<ceil_div(d.nd * P, 256), 256, 0, s>>>(part, g, P, d.nd, out);
+  k_dots_reduce<<<dim3(ceil_div(P, kDrC), d.nd), kDrC * kDrR, 0, s>>>(part, g, P, out);
   note_launch();
 }
 

@@ -132,7 +132,9 @@ __device__ __forceinline__ double fix_to_double(long long hi, long long lo, int 
 
 // Column exponent fields: F[c] = max over the rows of the exponent field of
 // |Re X[r][c]| and |Im X[r][c]| (F must be zeroed before).  blockIdx.y picks
-// X (0) or Y (1).
+// X (0) or Y (1).  Only the high words' exponent bits matter, so the maximum
+// is taken over them in integers; a warp walks rows with its lanes on the
+// columns (up to four each, in registers), four rows of loads in flight.
 __global__ void __launch_bounds__(256) k_col_expo(const cxd *__restrict__ X, int ldx, int mx, const cxd *__restrict__ Y,
                                                   int ldy, int my, int n, int rows_per_cta, int *FX, int *FY) {
   __shared__ int sm[kMaxM0];
@@ -141,20 +143,26 @@ __global__ void __launch_bounds__(256) k_col_expo(const cxd *__restrict__ X, int
   int *F = blockIdx.y ? FY : FX;
   for (int c = threadIdx.x; c < m; c += blockDim.x) sm[c] = 0;
   __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int r0 = blockIdx.x * rows_per_cta, r1 = min(n, r0 + rows_per_cta);
-  const long long cnt = r1 > r0 ? (long long)(r1 - r0) * m : 0;
-  int cur = -1, em = 0;
-  for (long long idx = threadIdx.x; idx < cnt; idx += blockDim.x) {
-    const int r = (int)(idx / m), c = (int)(idx - (long long)r * m);
-    if (c != cur) {
-      if (cur >= 0) atomicMax(&sm[cur], em);
-      cur = c;
-      em = 0;
+  int em[kMaxM0 / 32] = {0, 0, 0, 0};
+  for (int r = r0 + warp; r < r1; r += 4 * nw) {
+#pragma unroll
+    for (int q = 0; q < kMaxM0 / 32; ++q) {
+      const int c = lane + 32 * q;
+      if (c < m) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (r + u * nw < r1) {
+            const cxd v = M[(size_t)(r + u * nw) * ld + c];
+            em[q] = max(em[q], max(expo_field(v.re), expo_field(v.im)));
+          }
+      }
     }
-    const cxd v = M[(size_t)(r0 + r) * ld + c];
-    em = max(em, max(expo_field(v.re), expo_field(v.im)));
   }
-  if (cur >= 0) atomicMax(&sm[cur], em);
+#pragma unroll
+  for (int q = 0; q < kMaxM0 / 32; ++q)
+    if (lane + 32 * q < m) atomicMax(&sm[lane + 32 * q], em[q]);
   __syncthreads();
   for (int c = threadIdx.x; c < m; c += blockDim.x)
     if (sm[c]) atomicMax(&F[c], sm[c]);
@@ -377,7 +385,7 @@ void gram_tc(const cxd *X, int ldx, int mx, const cxd *Y, int ldy, int my, int n
   set_smem_attr(reinterpret_cast<const void *>(k_gram_tc), gram_tc_smem_bytes(), 0);
   int *FX = FXY, *FY = FXY + kMaxM0;
   cudaMemsetAsync(FXY, 0, 2 * kMaxM0 * sizeof(int), s);
-  const int erows = 1024;
+  const int erows = std::max(32, ceil_div(n, 608));  // enough CTAs for the chip, 32 rows at least
   k_col_expo<<<dim3(ceil_div(n, erows), 2), 256, 0, s>>>(X, ldx, mx, Y, ldy, my, n, erows, FX, FY);
   note_launch();
   int rpc = ceil_div(ceil_div(n, nchunks), kRows) * kRows;

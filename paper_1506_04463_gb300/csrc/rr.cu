@@ -15,40 +15,38 @@ __global__ void k_gamma_prep(int m, const cxd *BQ, const cxd *gam, const cxd *V,
   __shared__ int o[kMaxM0];
   __shared__ cxd g[kMaxM0];
   __shared__ cxd tcs[kMaxM0];
-  __shared__ int mt_s;
   const int tid = threadIdx.x, nt = blockDim.x;
-  if (tid == 0) {
-    int ms = 0;
-    if (have_prev) {
-      for (int i = 0; i < m; ++i) {
-        if (!prev_inside[i]) continue;
-        const cxd r2 = prev_rho[i] * prev_rho[i];
-        const cxd d = BQ[(size_t)i * m + i];
-        const double den = cabs(r2);
-        const double q = den > 0 ? cabs(r2 - d) / den : INFINITY;
-        if (!(q < mu)) ++ms;
-      }
-    }
-    st->m_s = ms;
-    for (int i = 0; i < m; ++i) o[i] = i;
-    for (int i = 1; i < m; ++i) {  // stable insertion sort, |gamma| descending
-      int key = o[i];
-      double kv = cabs(gam[key]);
-      int j = i - 1;
-      while (j >= 0 && cabs(gam[o[j]]) < kv) {
-        o[j + 1] = o[j];
-        --j;
-      }
-      o[j + 1] = key;
-    }
-    const double gmax = cabs(gam[o[0]]);
-    int mt = 0;
-    while (mt < m && cabs(gam[o[mt]]) >= eta * gmax && gmax > 0) ++mt;
-    mt_s = mt;
-    st->m_tilde = mt;
+  // moduli once, then every value finds its own place: the number of larger
+  // ones, and of equal ones before it (a stable sort, decreasing).  Moduli
+  // are compared as integers (the bits of non-negative doubles), since an FP64
+  // compare costs a warp 64 cycles; NaN goes last.
+  __shared__ long long key[kMaxM0];
+  double md = -1.0;
+  if (tid < m) {
+    md = cabs(gam[tid]);
+    key[tid] = md == md ? __double_as_longlong(md) : -1;
+  }
+  bool spur = false;
+  if (tid < m && have_prev && prev_inside[tid]) {
+    const cxd r2 = prev_rho[tid] * prev_rho[tid];
+    const cxd d = BQ[(size_t)tid * m + tid];
+    const double den = cabs(r2);
+    const double q = den > 0 ? cabs(r2 - d) / den : INFINITY;
+    spur = !(q < mu);
+  }
+  const int ms = __syncthreads_count(spur);
+  if (tid < m) {
+    int rank = 0;
+    for (int j = 0; j < m; ++j) rank += key[j] > key[tid] || (key[j] == key[tid] && j < tid);
+    o[rank] = tid;
   }
   __syncthreads();
-  const int mt = mt_s;
+  const double gmax = cabs(gam[o[0]]);
+  const int mt = __syncthreads_count(tid < m && md >= eta * gmax && gmax > 0);
+  if (tid == 0) {
+    st->m_s = ms;
+    st->m_tilde = mt;
+  }
   for (int b = tid; b < m; b += nt) {
     ord[b] = o[b];
     const cxd sq = csqrt(gam[o[b]]);
@@ -103,23 +101,37 @@ __global__ void k_cs_wnorm(int m, const cxd *BU, cxd *W, cxd *Wh) {
 }
 
 // Step 4.c: rho_a(lambda_i) = sum_j w_j / (z_j - lambda_i)   (eq. rational).
-__global__ void k_rho(int m, int ne, const cxd *z, const cxd *w, const cxd *lam, cxd *rho) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    cxd s = mk(0.0, 0.0);
-    for (int j = 0; j < ne; ++j) s = s + cdiv(w[j], z[j] - lam[i]);
-    rho[i] = s;
+// One warp per eigenvalue, a lane per node: the FP64 quotients (some 50
+// instructions of 64 cycles each) are formed side by side.
+__global__ void __launch_bounds__(32) k_rho(int ne, const cxd *z, const cxd *w, const cxd *lam, cxd *rho) {
+  const int i = blockIdx.x, lane = threadIdx.x;
+  const cxd l = lam[i];
+  cxd s = mk(0.0, 0.0);
+  for (int j = lane; j < ne; j += 32) s = s + cdiv(w[j], z[j] - l);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    s.re += __shfl_down_sync(0xffffffffu, s.re, o);
+    s.im += __shfl_down_sync(0xffffffffu, s.im, o);
   }
+  if (lane == 0) rho[i] = s;
 }
 
 // Y[:, i] /= ||y_i||, Yh[:, i] *= ||y_i|| (column scale of the Ritz vectors).
-__global__ void k_scale_pairs(cxd *Y, cxd *Yh, const double *nrm2, int m, size_t count) {
+// The root and the quotient of a column are formed once per CTA: by every
+// element they made the kernel FP64-bound (192 us at 90 000 x 64, of which
+// moving the 369 MB takes 54).
+__global__ void __launch_bounds__(256) k_scale_pairs(cxd *Y, cxd *Yh, const double *nrm2, int m, size_t count) {
+  __shared__ double sc[kMaxM0], inv[kMaxM0];
+  for (int c = threadIdx.x; c < m; c += blockDim.x) {
+    const double s = sqrt(nrm2[c]);
+    sc[c] = s > 0 ? s : 1.0;
+    inv[c] = s > 0 ? 1.0 / s : 1.0;
+  }
+  __syncthreads();
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
     const int c = (int)(e % m);
-    const double s = sqrt(nrm2[c]);
-    if (s > 0) {
-      Y[e] = (1.0 / s) * Y[e];
-      Yh[e] = s * Yh[e];
-    }
+    Y[e] = inv[c] * Y[e];
+    Yh[e] = sc[c] * Yh[e];
   }
 }
 
@@ -148,59 +160,48 @@ __device__ __forceinline__ bool inside_contour(cxd l, const RRParams &p) {
 // spurious test of the next iteration.
 __global__ void k_converge(RRParams p, int mt, const cxd *lam, const cxd *rho, const double *cn, double *res,
                            int *ord, cxd *prev_rho, int *prev_inside, RRStatus *st) {
-  __shared__ int ins[kMaxM0];
-  __shared__ double rs[kMaxM0];
-  const int tid = threadIdx.x;
-  for (int i = tid; i < mt; i += blockDim.x) {
-    const bool in = inside_contour(lam[i], p);
-    ins[i] = in;
-    double r = INFINITY;
+  __shared__ long long key[kMaxM0];  // bits of the residual (>= 0), or the largest integer outside
+  __shared__ double mxs[4];
+  const int tid = threadIdx.x, i = tid;  // 128 threads, mt <= 128
+  bool in = false;
+  double r = INFINITY;
+  if (i < mt) {
+    in = inside_contour(lam[i], p);
     if (in) {
       const double r1 = cn[i] / (p.alpha * cn[kMaxM0 + i]);
       const double r2 = cn[2 * kMaxM0 + i] / (p.alpha * cn[3 * kMaxM0 + i]);
       r = fmax(r1, r2);
       if (!(r == r)) r = INFINITY;
     }
-    rs[i] = r;
     res[i] = r;
     prev_rho[i] = rho[i];
     prev_inside[i] = in;
+    key[i] = in ? __double_as_longlong(r) : 0x7fffffffffffffffll;
   }
+  const int mr = __syncthreads_count(in);
+  // inside pairs by increasing residual, then the others by index: every pair
+  // counts the ones before it
+  const int m = mr - st->m_s;
+  int rank = 0;
+  if (i < mt) {
+    for (int j = 0; j < mt; ++j) rank += key[j] < key[i] || (key[j] == key[i] && j < i);
+    ord[rank] = i;
+  }
+  const bool low = in && rank < m;  // among the m lowest residuals
+  const bool bad = __syncthreads_or(low && !(r < p.eps));
+  const bool conv = m >= 1 && !bad;
+  const int below = __syncthreads_count(in && r < p.eps);
+  double mx = low ? r : 0.0;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((tid & 31) == 0) mxs[tid >> 5] = mx;
   __syncthreads();
   if (tid == 0) {
-    int mr = 0;
-    for (int i = 0; i < mt; ++i) mr += ins[i];
-    int k = 0;
-    for (int i = 0; i < mt; ++i)
-      if (ins[i]) ord[k++] = i;
-    for (int i = 1; i < k; ++i) {  // stable insertion sort by residual
-      int key = ord[i];
-      int j = i - 1;
-      while (j >= 0 && rs[ord[j]] > rs[key]) {
-        ord[j + 1] = ord[j];
-        --j;
-      }
-      ord[j + 1] = key;
-    }
-    for (int i = 0; i < mt; ++i)
-      if (!ins[i]) ord[k++] = i;
-    const int m = mr - st->m_s;
-    double mx = 0.0;
-    bool conv = m >= 1;
-    for (int i = 0; i < m && i < mr; ++i) {
-      mx = fmax(mx, rs[ord[i]]);
-      if (!(rs[ord[i]] < p.eps)) conv = false;
-    }
     // 5.d: on convergence every inside pair below eps is returned (at least m)
-    int mout = m > 0 ? m : 0;
-    if (conv) {
-      mout = 0;
-      while (mout < mr && rs[ord[mout]] < p.eps) ++mout;
-    }
     st->m_r = mr;
-    st->m = mout;
+    st->m = conv ? below : (m > 0 ? m : 0);
     st->conv = conv ? 1 : 0;
-    st->max_res = m >= 1 ? mx : INFINITY;
+    st->max_res = m >= 1 ? fmax(fmax(mxs[0], mxs[1]), fmax(mxs[2], mxs[3])) : INFINITY;
   }
 }
 
@@ -293,7 +294,7 @@ void launch_cs_wnorm(int m, const cxd *BU, cxd *W, cxd *Wh, cudaStream_t s) {
   note_launch();
 }
 void launch_rho(int m, int ne, const cxd *z, const cxd *w, const cxd *lam, cxd *rho, cudaStream_t s) {
-  k_rho<<<1, 128, 0, s>>>(m, ne, z, w, lam, rho);
+  k_rho<<<m, 32, 0, s>>>(ne, z, w, lam, rho);
   note_launch();
 }
 void launch_scale_pairs(cxd *Y, cxd *Yh, const double *nrm2, int m, int n, cudaStream_t s) {

@@ -10,6 +10,7 @@
 //  * csr transpose for the conjugate-transpose products A^H, B^H (eq. ql and
 //    the left residual of eq. res).
 #include "kernels.h"
+#include "reduce.cuh"
 
 template <bool CPLX>
 __device__ __forceinline__ void csr_fma(cxd &acc, const CsrView &M, int64_t k, const cxd &x) {
@@ -197,50 +198,53 @@ template int launch_multishift_residual_capped<double>(const CsrView &, const Cs
                                                        const cxd *, const cxd *, const cxd *, cxd *, cxd *, double *,
                                                        int, int, cudaStream_t);
 
-__global__ void k_residual_rel(const double *partial, int nparts, int P, int m, const double *bynorm2, int nsides,
-                               unsigned long long *maxbits) {
-  __shared__ double red[128];
-  double mx = 0.0;
-  const int sp = blockIdx.x * blockDim.x + threadIdx.x;
-  if (sp < nsides * P) {
-    const int side = sp / P, pair = sp - side * P;
-    const double *pb = partial + (size_t)side * nparts * P;
-    double s = 0.0;
-    for (int p = 0; p < nparts; ++p) s += pb[(size_t)p * P + pair];
+// One CTA per 4 (node, column) pairs, 64 threads a pair: at 1216 partials and
+// 2048 pairs this took 179 us with a thread per pair (a chain of 1216 loads);
+// spread out it is bound by reading the 20 MB of partials from L2.
+constexpr int kRelC = 4, kRelR = 64;
+__global__ void __launch_bounds__(kRelC *kRelR) k_residual_rel(const double *__restrict__ partial, int nparts, int P,
+                                                               int m, const double *bynorm2, int nsides,
+                                                               unsigned long long *maxbits) {
+  __shared__ double sm[kRelC * kRelR];
+  const int sp = blockIdx.x * kRelC + threadIdx.x % kRelC;
+  const bool ok = sp < nsides * P;
+  const int side = ok ? sp / P : 0, pair = ok ? sp - side * P : 0;
+  const double s = column_sum<kRelC, kRelR>(partial + (size_t)side * nparts * P, nparts, P, pair, ok, sm);
+  if (ok && threadIdx.x < kRelC) {
     const double d = bynorm2[side * m + pair % m];
     const double rel = d > 0 ? sqrt(s / d) : sqrt(s);
-    mx = (rel == rel) ? rel : INFINITY;
+    const double mx = (rel == rel) ? rel : INFINITY;
+    atomicMax(maxbits, (unsigned long long)__double_as_longlong(mx));
   }
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicMax(maxbits, (unsigned long long)__double_as_longlong(red[0]));
-}
-__global__ void k_residual_done(const unsigned long long *maxbits, double tol, double *maxrel, int *done) {
-  const double v = __longlong_as_double((long long)*maxbits);
-  *maxrel = v;
-  *done = v <= tol ? 1 : 0;
 }
 
 void launch_residual_check(const double *partial, int nparts, int ne, int m, const double *bynorm2, int nsides,
-                           double tol, double *d_maxrel, int *d_done, cudaStream_t s) {
+                           double *d_maxrel, cudaStream_t s) {
   // d_maxrel doubles as the atomic accumulator (bits of a non-negative double)
   unsigned long long *bits = reinterpret_cast<unsigned long long *>(d_maxrel);
   cudaMemsetAsync(bits, 0, sizeof(unsigned long long), s);
   const int total = nsides * ne * m;
-  k_residual_rel<<<ceil_div(total, 128), 128, 0, s>>>(partial, nparts, ne * m, m, bynorm2, nsides, bits);
-  note_launch();
-  k_residual_done<<<1, 1, 0, s>>>(bits, tol, d_maxrel, d_done);
+  k_residual_rel<<<ceil_div(total, kRelC), kRelC * kRelR, 0, s>>>(partial, nparts, ne * m, m, bynorm2, nsides, bits);
   note_launch();
 }
 
 // ---------------------------------------------------------------------------
 // single-shift products with per-column shift and column 1-norms
 // ---------------------------------------------------------------------------
-template <bool C1, bool C2>
+// |z|: the square root of |z|^2 where that neither over- nor underflows (by the
+// exponent field of the larger component, an integer test), else hypot, which
+// takes three times the FP64 instructions.
+__device__ __forceinline__ double modulus(cxd z) {
+  const int e = max(__double2hiint(z.re) & 0x7fffffff, __double2hiint(z.im) & 0x7fffffff) >> 20;
+  if (e > 1023 - 400 && e < 1023 + 400) return sqrt(fma(z.re, z.re, z.im * z.im));
+  return hypot(z.re, z.im);
+}
+
+// NORMS: also the per-CTA column 1-norms of Out and of M2 X (the residuals of
+// eq. res); the FP64 pipe bounds them, so products that don't need them (A U,
+// B Q) leave them out: 90 000 x 64, 5 entries a row, 490 us with both norms
+// by hypot.
+template <bool C1, bool C2, bool NORMS>
 __global__ void __launch_bounds__(256) k_spmm(CsrView M1, CsrView M2, int hasM2, const cxd *__restrict__ shift,
                                               const cxd *__restrict__ X, cxd *__restrict__ Out, int m,
                                               int rows_per_cta, double *p1, double *p2) {
@@ -268,11 +272,13 @@ __global__ void __launch_bounds__(256) k_spmm(CsrView M1, CsrView M2, int hasM2,
       }
       if (shift) cfms(acc, sh, bx);
       Out[(size_t)i * m + c] = acc;
-      a1 += cabs(acc);
-      a2 += cabs(bx);
+      if (NORMS) {
+        a1 += modulus(acc);
+        a2 += modulus(bx);
+      }
     }
   }
-  if (!p1) return;
+  if (!NORMS) return;
   r1[tid] = a1;
   r2[tid] = a2;
   __syncthreads();
@@ -294,7 +300,13 @@ int launch_spmm(const CsrView &M1, const CsrView *M2, const cxd *shift, const cx
   const int g = ceil_div(M1.n, rpc);
   CsrView M2v = M2 ? *M2 : M1;
   const bool c2 = M2 ? M2->cplx : false;
-#define SP_LAUNCH(A1, A2) k_spmm<A1, A2><<<g, 256, 0, s>>>(M1, M2v, M2 != nullptr, shift, X, Out, m, rpc, p1, p2)
+#define SP_LAUNCH(A1, A2)                                                                                        \
+  do {                                                                                                           \
+    if (p1)                                                                                                      \
+      k_spmm<A1, A2, true><<<g, 256, 0, s>>>(M1, M2v, M2 != nullptr, shift, X, Out, m, rpc, p1, p2);             \
+    else                                                                                                         \
+      k_spmm<A1, A2, false><<<g, 256, 0, s>>>(M1, M2v, M2 != nullptr, shift, X, Out, m, rpc, nullptr, nullptr);  \
+  } while (0)
   if (M1.cplx) {
     if (c2) SP_LAUNCH(true, true); else SP_LAUNCH(true, false);
   } else {
@@ -305,15 +317,18 @@ int launch_spmm(const CsrView &M1, const CsrView *M2, const cxd *shift, const cx
   return g;
 }
 
-__global__ void k_reduce_parts(const double *parts, int nparts, int m, double *out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int p = 0; p < nparts; ++p) s += parts[(size_t)p * m + c];
-    out[c] = s;
-  }
+// out[c] = sum of the partials of column c: one CTA per 4 columns.  1216
+// partials of 64 columns: 100 us with a thread per column.
+constexpr int kRpC = 4, kRpR = 64;
+__global__ void __launch_bounds__(kRpC *kRpR) k_reduce_parts(const double *__restrict__ parts, int nparts, int m,
+                                                             double *out) {
+  __shared__ double sm[kRpC * kRpR];
+  const int c = blockIdx.x * kRpC + threadIdx.x % kRpC;
+  const double s = column_sum<kRpC, kRpR>(parts, nparts, m, c, c < m, sm);
+  if (c < m && threadIdx.x < kRpC) out[c] = s;
 }
 void launch_reduce_parts(const double *parts, int nparts, int m, double *out, cudaStream_t s) {
-  k_reduce_parts<<<ceil_div(m, 256), 256, 0, s>>>(parts, nparts, m, out);
+  k_reduce_parts<<<ceil_div(m, kRpC), kRpC * kRpR, 0, s>>>(parts, nparts, m, out);
   note_launch();
 }
 
