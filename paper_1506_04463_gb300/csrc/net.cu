@@ -7,21 +7,27 @@
 // Activations are channel-last (image, y, x, 32 channels): 64 bytes a pixel.
 // Weights W_l[tap][c_in][c_out], tap = 3*dy + dx for the offset (dy-1, dx-1).
 //
-// k_conv3x3_tc: the convolution as an implicit GEMM on the tensor cores.
-// A CTA of 128 threads takes tiles of 128 consecutive pixels; per tile
-//   D (128 pixels x 32 out-channels, FP32, in tensor memory)
-//     = A (128 x 288: the nine shifted 32-channel neighbours of each pixel)
-//     x B (288 x 32: the weights),
-// with A and B in shared memory in the canonical no-swizzle K-major layout
-// (8-row x 16-byte core matrices; LBO = 128 B between core matrices along K,
-// SBO = 36 * 128 B between 8-row groups), issued as 18 tcgen05.mma
-// (M = 128, N = 32, K = 16, kind::f16 with BF16 operands) by one thread and
-// committed to an mbarrier; every warp then reads its 32 rows of D with
+// The convolution (forward, and backward with the weights mirrored and their
+// channel axes swapped) and the weight gradient both run on the tensor cores.
+// In shared memory an operand is kept as [channel chunk of 8][pixel], 16 bytes
+// an entry: eight consecutive entries are a core matrix whatever pixel they
+// start at, so the nine taps are the same pixels read from other start
+// addresses, and nothing is copied nine times.
+//
+// Pixels are numbered by position q: rows of N + 1, the last one a pad that
+// reads as zero, so that the left and right neighbours of q are q - 1 and
+// q + 1 also at the ends of a row.  The neighbours above and below come from
+// segments of their own (rows y - 1, y, y + 1), zero outside the image.
+//
+// k_conv3x3_tc: a CTA takes tiles of 128 positions; D (128 x 32, FP32, in
+// tensor memory) = sum over the taps of A_tap (128 x 32) W_tap (32 x 32), 18
+// tcgen05.mma (M = 128, N = 32, K = 16); each warp reads its 32 rows with
 // tcgen05.ld and applies the epilogue (bias, ReLU, or the ReLU mask of the
-// backward pass) before storing BF16 (and optionally FP32) results.
-// The backward data pass is the same kernel with the weights flipped and
-// their channel axes swapped; the weight gradient is a CUDA-core reduction
-// over pixels (per-CTA partials, fixed-order sum).
+// backward pass).
+// k_conv_wgrad: dW[tap][ci][co] = sum_p a[p + off(tap)][ci] g[p][co]: three
+// GEMMs (dy) of M = 3 dx x 32 ci (and a row of ones for the bias gradient),
+// N = 32, K = positions, accumulated in tensor memory; per-CTA partials are
+// summed in FP64 in fixed order.
 #include <algorithm>
 #include <cuda_bf16.h>
 #include "kernels.h"
@@ -31,29 +37,31 @@ namespace {
 
 constexpr int kC = 32;               // channels
 constexpr int kK = 9 * kC;           // GEMM depth: 288
-constexpr int kTile = 128;           // pixels per tile (GEMM M)
-constexpr int kLBO = 128;            // bytes between core matrices along K
-constexpr int kSBO = (kK / 8) * 128; // bytes between 8-row groups: 4608
-constexpr int kAB = kTile * kK * 2;  // A tile bytes: 73728
-constexpr int kBB = kC * kK * 2;     // weight bytes: 18432
+constexpr int kTile = 128;           // positions per tile (GEMM M)
+constexpr int kSegPix = kTile + 2;   // staged pixels of a row segment
+// chunk strides of 32 bytes modulo 128: the 16-byte stores of two pixels x four
+// chunks that a quarter-warp issues together fall on distinct banks
+constexpr int kChunkA = kSegPix * 16;        // 2080
+constexpr int kSegBytes = 4 * kChunkA;
+constexpr int kChunkB = kK * 16 + 32;        // 4640
+constexpr int kAB = 3 * kSegBytes;           // three row segments: 24960
+constexpr int kBB = 4 * kChunkB;             // weights: 18560
 
 using tc::smem_u32;
 using tc::smem_desc;
 using tc::mbar_init;
 using tc::mbar_wait;
-constexpr uint32_t kIdesc = tc::idesc_bf16(kTile, kC);
-
-// byte offset of element (row, k) in a canonical K-major no-swizzle operand
-__device__ __forceinline__ int canon_off(int row, int k) {
-  return (row >> 3) * kSBO + (k >> 3) * kLBO + (row & 7) * 16 + (k & 7) * 2;
-}
+constexpr uint32_t kIdesc = tc::idesc_bf16(kTile, kC, false, true);  // A K-major, W as stored (c_out fastest)
 
 }  // namespace
 
 // out[p][co] = epilogue(sum_{tap, ci} W[tap][ci][co] in[p + off(tap)][ci])
 // epilogue: + bias[co] (if bias), relu (if relu), * (mask[p][co] > 0) (if mask);
 // stored as BF16 to out (if out) and FP32 to outf (if outf).
-__global__ void __launch_bounds__(128, 2) k_conv3x3_tc(const __nv_bfloat16 *__restrict__ in,
+// Bound by moving the activations (64 bytes a pixel in, 64 out).  With an
+// im2col copy of every pixel into nine taps and the weights scattered two bytes
+// at a time, 196 608 pixels took 38 us a layer; the shared segments stage three.
+__global__ void __launch_bounds__(128, 5) k_conv3x3_tc(const __nv_bfloat16 *__restrict__ in,
                                                        const __nv_bfloat16 *__restrict__ W,
                                                        const float *__restrict__ bias,
                                                        const __nv_bfloat16 *__restrict__ mask, int relu,
@@ -65,63 +73,60 @@ __global__ void __launch_bounds__(128, 2) k_conv3x3_tc(const __nv_bfloat16 *__re
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kAB + kBB);
   uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + kAB + kBB + 16);
   const int tid = threadIdx.x, warp = tid >> 5;
-  // weights -> canonical B layout (row = out-channel n, k = tap*32 + ci)
-  for (int e = tid; e < kK * (kC / 8); e += blockDim.x) {
-    const int k = e / (kC / 8), n8 = (e % (kC / 8)) * 8;  // 8 consecutive out-channels of one k
-    const int tap = k / kC, ci = k % kC;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const __nv_bfloat16 v = W[((size_t)tap * kC + ci) * kC + n8 + q];
-      *reinterpret_cast<__nv_bfloat16 *>(Bs + canon_off(n8 + q, k)) = v;
-    }
-  }
+  // weights: [chunk of 8 out-channels][k = tap*32 + ci]
+  for (int e = tid; e < kK * 4; e += 128)
+    *reinterpret_cast<uint4 *>(Bs + (e & 3) * kChunkB + (e >> 2) * 16) =
+        *reinterpret_cast<const uint4 *>(W + (size_t)(e >> 2) * kC + (e & 3) * 8);
   if (tid == 0) mbar_init(bar, 1);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_u32(tslot)));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (warp == 0) tc::tmem_alloc(tslot, 32);
+  tc::fence_smem();
+  tc::fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  tc::fence_after();
   const uint32_t tmem = *tslot;
-  const long long npix = (long long)nimg * N * N;
-  const long long ntiles = (npix + kTile - 1) / kTile;
+  const int wd = N + 1;
+  const long long npos = (long long)nimg * N * wd;
+  const long long ntiles = (npos + kTile - 1) / kTile;
   uint32_t phase = 0;
   bool ok = true;
   for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-    // ---- im2col of this thread's pixel into the canonical A layout ----
-    const long long p = t * kTile + tid;
-    int img = 0, y = 0, x = 0;
-    const bool live = p < npix;
-    if (live) {
-      img = (int)(p / ((long long)N * N));
-      const int rem = (int)(p - (long long)img * N * N);
-      y = rem / N;
-      x = rem - y * N;
-    }
+    // ---- rows y - 1, y, y + 1 of positions q0 - 1 .. q0 + 128 ----
+    const long long qb = t * kTile - 1;  // first staged position (-1: a pad)
+    const int rb = qb < 0 ? -1 : (int)(qb / wd), xb = qb < 0 ? N : (int)(qb - (long long)rb * wd);
+    const int yb = rb < 0 ? -1 : rb % N;
+    const int live_px = (int)min((long long)kSegPix, npos - qb);
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-      const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-      const bool inb = live && yy >= 0 && yy < N && xx >= 0 && xx < N;
-      const uint4 *src = reinterpret_cast<const uint4 *>(in + (((size_t)img * N + (inb ? yy : 0)) * N +
-                                                               (inb ? xx : 0)) * kC);
+    for (int it = 0; it < (kSegPix * 4 + 127) / 128; ++it) {
+      const int e = tid + it * 128;
+      if (e < kSegPix * 4) {
+        const int i = e >> 2, ch = e & 3;
+        const int dr = (xb + i) / wd, x = xb + i - dr * wd;
+        const int y = (yb + dr) % N;  // not used when the position is a pad
+        const bool px = x < N && i < live_px;
+        const __nv_bfloat16 *src = in + ((long long)(rb + dr) * N + x) * kC + ch * 8;
+        uint4 v[3];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 v = inb ? src[q] : make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4 *>(As + canon_off(tid, tap * kC + q * 8)) = v;
+        for (int dy = 0; dy < 3; ++dy) {
+          const bool inb = px && y + dy - 1 >= 0 && y + dy - 1 < N;
+          v[dy] = inb ? *reinterpret_cast<const uint4 *>(src + (long long)(dy - 1) * N * kC) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+          *reinterpret_cast<uint4 *>(As + dy * kSegBytes + ch * kChunkA + i * 16) = v[dy];
       }
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc::fence_smem();
     __syncthreads();
     // ---- 18 MMAs, K = 16 each ----
     if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc::fence_after();
       const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
 #pragma unroll
-      for (int s = 0; s < kK / 16; ++s)
-        tc::mma(tmem, smem_desc(a0 + s * 2 * kLBO, kLBO, kSBO), smem_desc(b0 + s * 2 * kLBO, kLBO, kSBO), kIdesc,
-                s > 0);
+      for (int s = 0; s < kK / 16; ++s) {
+        const int tap = s >> 1;
+        tc::mma(tmem, smem_desc(a0 + (tap / 3) * kSegBytes + (tap % 3) * 16 + (s & 1) * 2 * kChunkA, kChunkA, 128),
+                smem_desc(b0 + s * 256, 128, kChunkB), kIdesc, s > 0);
+      }
       tc::commit(bar);
     }
     // the CTA agrees on the outcome of the bounded wait, so that every thread
@@ -132,11 +137,13 @@ __global__ void __launch_bounds__(128, 2) k_conv3x3_tc(const __nv_bfloat16 *__re
       ok = false;
     }
     phase ^= 1;
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // ---- epilogue: warp w holds rows (pixels) 32w .. 32w+31 ----
+    tc::fence_after();
+    // ---- epilogue: warp w holds rows (positions) 32w .. 32w+31 ----
     float v[32];
     tc::ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
-    if (live) {
+    const int dr = (xb + 1 + tid) / wd, x = xb + 1 + tid - dr * wd;
+    if (x < N && tid + 1 < live_px) {
+      const size_t p = (size_t)(rb + dr) * N + x;
       if (bias) {
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] += bias[k];
@@ -146,12 +153,20 @@ __global__ void __launch_bounds__(128, 2) k_conv3x3_tc(const __nv_bfloat16 *__re
         for (int k = 0; k < 32; ++k) v[k] = fmaxf(v[k], 0.f);
       }
       if (mask) {
-        const __nv_bfloat16 *mk_ = mask + (size_t)p * kC;
+        const uint4 *mk_ = reinterpret_cast<const uint4 *>(mask + p * kC);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = __bfloat162float(mk_[k]) > 0.f ? v[k] : 0.f;
+        for (int q = 0; q < 4; ++q) {
+          const uint4 m4 = mk_[q];
+          const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            v[q * 8 + 2 * u] = __uint_as_float(mw[u] << 16) > 0.f ? v[q * 8 + 2 * u] : 0.f;
+            v[q * 8 + 2 * u + 1] = __uint_as_float(mw[u] & 0xffff0000u) > 0.f ? v[q * 8 + 2 * u + 1] : 0.f;
+          }
+        }
       }
       if (out) {
-        uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)p * kC);
+        uint4 *dst = reinterpret_cast<uint4 *>(out + p * kC);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           __nv_bfloat162 h[4];
@@ -161,16 +176,16 @@ __global__ void __launch_bounds__(128, 2) k_conv3x3_tc(const __nv_bfloat16 *__re
         }
       }
       if (outf) {
-        float4 *dst = reinterpret_cast<float4 *>(outf + (size_t)p * kC);
+        float4 *dst = reinterpret_cast<float4 *>(outf + p * kC);
 #pragma unroll
         for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc::fence_before();
     __syncthreads();
   }
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem));
+  if (warp == 0) tc::tmem_free(tmem, 32);
 }
 
 // Weights of the adjoint convolution: Wt[tap'][co][ci] = W[tap][ci][co] with
@@ -183,78 +198,187 @@ __global__ void k_conv_adjoint_weights(const __nv_bfloat16 *W, __nv_bfloat16 *Wt
 }
 
 // Weight and bias gradients of one layer: dW[tap][ci][co] = sum_p
-// a[p + off(tap)][ci] g[p][co], db[co] = sum_p g[p][co].  Each CTA reduces a
-// contiguous chunk of pixels into its own partial (thread = (tap, ci), 32
-// accumulators); k_net_reduce sums the partials in CTA order.
-constexpr int kGradPix = 64;
-__global__ void __launch_bounds__(288) k_conv_wgrad(const __nv_bfloat16 *__restrict__ a,
-                                                    const __nv_bfloat16 *__restrict__ g, int nimg, int N,
-                                                    long long pix_per_cta, float *__restrict__ part) {
-  __shared__ float gs[kGradPix][kC];
-  const int tid = threadIdx.x;  // tid = tap * 32 + ci
-  const int tap = tid / kC, ci = tid % kC;
-  const long long npix = (long long)nimg * N * N;
-  const long long p0 = blockIdx.x * pix_per_cta, p1 = min(npix, p0 + pix_per_cta);
-  float acc[kC];
-#pragma unroll
-  for (int k = 0; k < kC; ++k) acc[k] = 0.f;
-  float bacc = 0.f;
-  for (long long pb = p0; pb < p1; pb += kGradPix) {
-    const int cnt = (int)min((long long)kGradPix, p1 - pb);
-    __syncthreads();
-    for (int e = tid; e < kGradPix * kC; e += blockDim.x) {
-      const int r = e / kC, c = e % kC;
-      gs[r][c] = r < cnt ? __bfloat162float(g[(size_t)(pb + r) * kC + c]) : 0.f;
-    }
-    __syncthreads();
-    for (int r = 0; r < cnt; ++r) {
-      const long long p = pb + r;
-      const int img = (int)(p / ((long long)N * N));
-      const int rem = (int)(p - (long long)img * N * N);
-      const int y = rem / N, x = rem - (rem / N) * N;
-      const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-      if (yy < 0 || yy >= N || xx < 0 || xx >= N) continue;
-      const float av = __bfloat162float(a[(((size_t)img * N + yy) * N + xx) * kC + ci]);
-#pragma unroll
-      for (int k = 0; k < kC; ++k) acc[k] = fmaf(av, gs[r][k], acc[k]);
-    }
-    if (tid < kC)
-      for (int r = 0; r < cnt; ++r) bacc += gs[r][tid];
+// a[p + off(tap)][ci] g[p][co], db[co] = sum_p g[p][co] (see the file comment).
+// A CTA of 256 threads takes stages of 64 positions, two in flight: the pixels
+// of the three row segments are stored at the three dx shifts (chunks
+// (dy*3 + dx)*4 + c, MN-major: 8 channels an entry), the gradient once; one
+// thread issues 3 dy x 4 MMAs (M = 128, N = 32, K = 16).  Rows 96..127 of a
+// product belong to the next dy's chunks and are not read, except row 96 of
+// dy = 2, whose chunk holds ones: the bias gradient.
+// On the CUDA cores (a thread per (tap, ci), 32 accumulators, every pixel's
+// gradient broadcast from shared memory) 196 608 pixels took 2.28 ms a layer.
+constexpr int kGPix = 64;
+constexpr int kGChunk = kGPix * 16 + 32;
+constexpr int kGA = 40 * kGChunk;
+constexpr int kGBuf = kGA + 4 * kGChunk;
+constexpr uint32_t kIdescW = tc::idesc_bf16(128, kC, true, true);
+__global__ void __launch_bounds__(256, 2) k_conv_wgrad(const __nv_bfloat16 *__restrict__ a,
+                                                       const __nv_bfloat16 *__restrict__ g, int nimg, int N,
+                                                       float *__restrict__ part, int *err) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + 2 * kGBuf);
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + 2 * kGBuf + 16);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int e = tid; e < 2 * 4 * kGPix; e += 256) {
+    const int b = e / (4 * kGPix), ch = e / kGPix % 4, k = e % kGPix;
+    *reinterpret_cast<uint4 *>(smem + b * kGBuf + (36 + ch) * kGChunk + k * 16) =
+        make_uint4(ch == 0 ? 0x3F80u : 0u, 0, 0, 0);  // BF16 one in the chunk's first channel
   }
-  float *o = part + (size_t)blockIdx.x * (9 * kC * kC + kC);
+  if (tid == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+  }
+  if (warp == 0) tc::tmem_alloc(tslot, 128);
+  tc::fence_smem();
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = *tslot;
+  const int wd = N + 1;
+  const long long npos = (long long)nimg * N * wd;
+  const long long ntiles = (npos + kGPix - 1) / kGPix;
+  bool ok = true;
+  int it = 0;
+  for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
+    const int b = it & 1;
+    unsigned char *Ab = smem + b * kGBuf, *Gb = Ab + kGA;
+    if (it >= 2) {  // the products that read this buffer are done
+      const bool w = mbar_wait(&bar[b], ((it >> 1) - 1) & 1);
+      if (__syncthreads_or(!w)) {
+        ok = false;
+        break;
+      }
+    }
+    const long long qb = t * kGPix - 1;
+    const int rb = qb < 0 ? -1 : (int)(qb / wd), xb = qb < 0 ? N : (int)(qb - (long long)rb * wd);
+    const int yb = rb < 0 ? -1 : rb % N;
+    const int live_px = (int)min((long long)(kGPix + 2), npos - qb);
 #pragma unroll
-  for (int k = 0; k < kC; ++k) o[(size_t)tid * kC + k] = acc[k];
-  if (tid < kC) o[9 * kC * kC + tid] = bacc;
+    for (int r = 0; r < 2; ++r) {
+      const int e = tid + r * 256;
+      if (e < (kGPix + 2) * 4) {
+        const int i = e >> 2, ch = e & 3;
+        const int dr = (xb + i) / wd, x = xb + i - dr * wd;
+        const int y = (yb + dr) % N;
+        const bool px = x < N && i < live_px;
+        const long long off = ((long long)(rb + dr) * N + x) * kC + ch * 8;
+        uint4 v[3], gv = make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const bool inb = px && y + dy - 1 >= 0 && y + dy - 1 < N;
+          v[dy] = inb ? *reinterpret_cast<const uint4 *>(a + off + (long long)(dy - 1) * N * kC)
+                      : make_uint4(0, 0, 0, 0);
+        }
+        if (px && i >= 1 && i <= kGPix) gv = *reinterpret_cast<const uint4 *>(g + off);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+          for (int dx = 0; dx < 3; ++dx)  // staged pixel i is position k + dx - 1 + 1 of copy dx
+            if (i - dx >= 0 && i - dx < kGPix)
+              *reinterpret_cast<uint4 *>(Ab + ((dy * 3 + dx) * 4 + ch) * kGChunk + (i - dx) * 16) = v[dy];
+        if (i >= 1 && i <= kGPix) *reinterpret_cast<uint4 *>(Gb + ch * kGChunk + (i - 1) * 16) = gv;
+      }
+    }
+    tc::fence_smem();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after();
+      const uint32_t a0 = smem_u32(Ab), g0 = smem_u32(Gb);
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int k = 0; k < kGPix / 16; ++k)
+          tc::mma(tmem + 32 * dy, smem_desc(a0 + dy * 12 * kGChunk + k * 256, 128, kGChunk),
+                  smem_desc(g0 + k * 256, 128, kGChunk), kIdescW, (it > 0 || k > 0) ? 1u : 0u);
+      tc::commit(&bar[b]);
+    }
+  }
+  // the last two stages' products (waited for also after a timeout, bounded,
+  // before the shared and tensor memory they use is given up)
+  for (int j = max(0, it - 2); j < it; ++j)
+    if (!mbar_wait(&bar[j & 1], (j >> 1) & 1)) ok = false;
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) atomicOr(err, DEVERR_TIMEOUT);
+  }
+  tc::fence_after();
+  float *o = part + (size_t)blockIdx.x * (9 * kC * kC + kC);
+  const int dx = warp & 3;  // the quarter of tensor-memory lanes this warp can read
+#pragma unroll
+  for (int dy = 0; dy < 3; ++dy) {
+    if ((dy == 2) != (warp >= 4)) continue;  // warps 0-3: dy = 0, 1; warps 4-7: dy = 2
+    float v[32];
+    tc::ld32(tmem + ((uint32_t)(dx * 32) << 16) + 32 * dy, v);
+    float4 *dst = nullptr;
+    if (dx < 3) dst = reinterpret_cast<float4 *>(o + ((size_t)(dy * 3 + dx) * kC + lane) * kC);
+    if (dx == 3 && dy == 2 && lane == 0) dst = reinterpret_cast<float4 *>(o + 9 * kC * kC);
+    if (dst) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc::fence_after();
+    tc::tmem_free(tmem, 128);
+  }
 }
 
-__global__ void k_net_reduce(const float *part, int nparts, int count, float *out) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int p = 0; p < nparts; ++p) s += part[(size_t)p * count + e];
-    out[e] = (float)s;
+// out[e] = sum of the partials in FP64: a CTA takes 8 outputs, 32 threads each.
+__global__ void __launch_bounds__(256) k_net_reduce(const float *__restrict__ part, int nparts, int count, float *out) {
+  __shared__ double sm[256];
+  const int e = blockIdx.x * 8 + (threadIdx.x & 7), r = threadIdx.x >> 3;
+  double s = 0.0;
+  if (e < count)
+    for (int p = r; p < nparts; p += 32) s += part[(size_t)p * count + e];
+  sm[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = 16; o; o >>= 1) {
+    if (r < o) sm[threadIdx.x] += sm[threadIdx.x + o * 8];
+    __syncthreads();
   }
+  if (e < count && r == 0) out[e] = (float)sm[threadIdx.x];
 }
 
 // Loss of the first cout channels against the FP32 target and its gradient
 // g = 2 (out - t) / count as BF16 (other channels zero); loss summed in FP64.
-__global__ void k_net_loss_grad(const float *__restrict__ out, const float *__restrict__ target, int cout,
-                                long long npix, __nv_bfloat16 *__restrict__ g, double *loss) {
+// A thread takes a pixel, so that the FP64 instructions of a warp serve 32
+// pixels' channels instead of the 32 channels of one pixel (87 us before at
+// 196 608 pixels with two channels).
+__global__ void __launch_bounds__(256) k_net_loss_grad(const float *__restrict__ out, const float *__restrict__ target,
+                                                       int cout, long long npix, __nv_bfloat16 *__restrict__ g,
+                                                       double *loss) {
+  __shared__ double red[8];
   double local = 0.0;
   const double inv = 1.0 / ((double)npix * cout);
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < npix * kC;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long p = e / kC;
-    const int c = (int)(e - p * kC);
-    float gv = 0.f;
-    if (c < cout) {
-      const float d = out[e] - target[p * cout + c];
-      local += (double)d * d;
-      gv = (float)(2.0 * d * inv);
+  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < npix;
+       p += (long long)gridDim.x * blockDim.x) {
+    uint4 *gp = reinterpret_cast<uint4 *>(g + p * kC);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      __nv_bfloat16 h[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int c = q * 8 + u;
+        float gv = 0.f;
+        if (c < cout) {
+          const float d = out[p * kC + c] - target[p * cout + c];
+          local += (double)d * d;
+          gv = (float)(2.0 * d * inv);
+        }
+        h[u] = __float2bfloat16(gv);
+      }
+      gp[q] = *reinterpret_cast<uint4 *>(h);
     }
-    g[e] = __float2bfloat16(gv);
   }
   for (int o = 16; o; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, local * inv);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = local;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += red[w];
+    atomicAdd(loss, s * inv);
+  }
 }
 
 // Adam step on FP32 master parameters; BF16 copy of the weights for the
@@ -271,9 +395,26 @@ __global__ void k_net_adam(float *w, const float *grad, float *m1, float *m2, in
   }
 }
 
-__global__ void k_to_bf16(const float *x, __nv_bfloat16 *y, long long count) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count; e += (long long)gridDim.x * blockDim.x)
-    y[e] = __float2bfloat16(x[e]);
+// count a multiple of 8 (whole channel groups), 32 bytes in and 16 out a thread;
+// vec = 0: x is not on a 16-byte boundary (a caller's view), scalar loads
+__global__ void k_to_bf16(const float *x, __nv_bfloat16 *y, long long count, int vec) {
+  const float4 *x4 = reinterpret_cast<const float4 *>(x);
+  uint4 *y4 = reinterpret_cast<uint4 *>(y);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count / 8;
+       e += (long long)gridDim.x * blockDim.x) {
+    float4 u, v;
+    if (vec) {
+      u = x4[2 * e];
+      v = x4[2 * e + 1];
+    } else {
+      const float *xs = x + 8 * e;
+      u = make_float4(xs[0], xs[1], xs[2], xs[3]);
+      v = make_float4(xs[4], xs[5], xs[6], xs[7]);
+    }
+    __nv_bfloat162 h[4] = {__floats2bfloat162_rn(u.x, u.y), __floats2bfloat162_rn(u.z, u.w),
+                           __floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
+    y4[e] = *reinterpret_cast<uint4 *>(h);
+  }
 }
 __global__ void k_bf16_to_f32(const __nv_bfloat16 *x, float *y, long long count) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count; e += (long long)gridDim.x * blockDim.x)
@@ -459,8 +600,8 @@ cudaError_t launch_conv3x3_tc(const void *in, const void *W, const float *bias, 
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const long long ntiles = ((long long)nimg * N * N + kTile - 1) / kTile;
-  long long g = (long long)sms * 2;
+  const long long ntiles = ((long long)nimg * N * (N + 1) + kTile - 1) / kTile;
+  long long g = (long long)sms * 5;  // resident CTAs (43.6 KB of shared memory, 128 threads)
   if (g > ntiles) g = ntiles;
   if (g < 1) g = 1;
   k_conv3x3_tc<<<(unsigned)g, kTile, conv_tc_smem_bytes(), s>>>(
@@ -475,26 +616,31 @@ void launch_conv_adjoint_weights(const void *W, void *Wt, cudaStream_t s) {
   note_launch();
 }
 
-int conv_wgrad_parts(long long npix) {
-  long long p = (npix + 4095) / 4096;
-  if (p > 1216) p = 1216;
-  return (int)(p < 1 ? 1 : p);
+static int wgrad_parts(int nimg, int N) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long tiles = ((long long)nimg * N * (N + 1) + kGPix - 1) / kGPix;
+  return (int)std::min<long long>(tiles, 2 * sms);  // two resident CTAs an SM
 }
 
-void launch_conv_wgrad(const void *a, const void *g, int nimg, int N, float *part, float *dWb, cudaStream_t s) {
-  const long long npix = (long long)nimg * N * N;
-  const int parts = conv_wgrad_parts(npix);
-  const long long per = (npix + parts - 1) / parts;
-  k_conv_wgrad<<<parts, 288, 0, s>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)g, nimg, N, per, part);
+cudaError_t launch_conv_wgrad(const void *a, const void *g, int nimg, int N, float *part, float *dWb, int *err,
+                              cudaStream_t s) {
+  const size_t smem = 2 * kGBuf + 64;
+  cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int parts = wgrad_parts(nimg, N);
+  k_conv_wgrad<<<parts, 256, smem, s>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)g, nimg, N, part, err);
   note_launch();
   const int count = 9 * kC * kC + kC;
-  k_net_reduce<<<ceil_div(count, 256), 256, 0, s>>>(part, parts, count, dWb);
+  k_net_reduce<<<ceil_div(count, 8), 256, 0, s>>>(part, parts, count, dWb);
   note_launch();
+  return cudaGetLastError();
 }
 
 void launch_net_loss_grad(const float *out, const float *target, int cout, long long npix, void *g, double *loss,
                           cudaStream_t s) {
-  k_net_loss_grad<<<grid_for((size_t)npix * kC), 256, 0, s>>>(out, target, cout, npix, (__nv_bfloat16 *)g, loss);
+  k_net_loss_grad<<<grid_for((size_t)npix), 256, 0, s>>>(out, target, cout, npix, (__nv_bfloat16 *)g, loss);
   note_launch();
 }
 
@@ -506,7 +652,7 @@ void launch_net_adam(float *w, const float *grad, float *m1, float *m2, int coun
 }
 
 void launch_to_bf16(const float *x, void *y, long long count, cudaStream_t s) {
-  k_to_bf16<<<grid_for((size_t)count), 256, 0, s>>>(x, (__nv_bfloat16 *)y, count);
+  k_to_bf16<<<grid_for((size_t)count / 8), 256, 0, s>>>(x, (__nv_bfloat16 *)y, count, (reinterpret_cast<uintptr_t>(x) & 15) == 0);
   note_launch();
 }
 void launch_bf16_to_f32(const void *x, float *y, long long count, cudaStream_t s) {
@@ -659,7 +805,7 @@ feast_nh_status feast_nh_net_create(feast_nh_net **out, int32_t layers, int32_t 
   n->outf = nalloc<float>(n, pix * kC * sizeof(float), ok);
   n->g0 = nalloc<__nv_bfloat16>(n, pix * kC * 2, ok);
   n->g1 = nalloc<__nv_bfloat16>(n, pix * kC * 2, ok);
-  n->wpart = nalloc<float>(n, (size_t)conv_wgrad_parts((long long)pix) * kLayerP * sizeof(float), ok);
+  n->wpart = nalloc<float>(n, (size_t)wgrad_parts(max_images, N) * kLayerP * sizeof(float), ok);
   n->dloss = nalloc<double>(n, sizeof(double), ok);
   n->derr = nalloc<int>(n, sizeof(int), ok);
   if (!ok) {
@@ -723,7 +869,12 @@ static feast_nh_status net_backward(feast_nh_net *n, __nv_bfloat16 *g, int nimg,
   cudaStream_t s = n->s;
   __nv_bfloat16 *gn = (g == n->g0) ? n->g1 : n->g0;
   for (int l = n->L - 1; l >= 0; --l) {
-    launch_conv_wgrad(n->act[l], g, nimg, n->N, n->wpart, n->grad + (size_t)l * kLayerP, s);
+    const cudaError_t ew =
+        launch_conv_wgrad(n->act[l], g, nimg, n->N, n->wpart, n->grad + (size_t)l * kLayerP, n->derr, s);
+    if (ew != cudaSuccess) {
+      n->err = std::string("network backward: ") + cudaGetErrorString(ew);
+      return FEAST_NH_ECUDA;
+    }
     if (l > 0) {
       launch_conv_adjoint_weights(n->wb + (size_t)l * kLayerW, n->wt, s);
       const cudaError_t e = launch_conv3x3_tc(g, n->wt, nullptr, n->act[l], 0, gn, nullptr, nimg, n->N, n->derr, s);

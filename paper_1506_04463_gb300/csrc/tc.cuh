@@ -1,8 +1,10 @@
 // Thin wrappers over the sm_103a tensor-core (tcgen05), mbarrier and async-
 // proxy instructions used by the project's tensor-core kernels.  Operands are
-// staged in shared memory in the canonical no-swizzle K-major layout: 8-row x
-// 16-byte core matrices, LBO = distance between core matrices along K, SBO =
-// distance between 8-row groups.
+// staged in shared memory in the canonical no-swizzle layouts: core matrices of
+// 8 rows of 16 bytes, LBO = distance between core matrices along K, SBO =
+// distance between them along M or N.  K-major: a row is one M (N) index, its
+// 16 bytes are 8 consecutive k; MN-major: a row is one k, its 16 bytes are 8
+// consecutive M (N) indices.
 #pragma once
 #include <cstdint>
 
@@ -26,8 +28,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 // Instruction descriptor of kind::f16 with BF16 A and B (both K-major) and an
 // FP32 accumulator: D type bits 4-5 = 1, A type bits 7-9 = 1, B type bits
 // 10-12 = 1, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// a_mn / b_mn: that operand is MN-major (its M or N index runs within the
+// 16-byte rows of the core matrices) instead of K-major (bits 15 and 16).
+constexpr uint32_t idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
