@@ -55,6 +55,16 @@ template <typename T> HD cx<T> cdiv(cx<T> a, cx<T> b) {
     return mk((a.re * r + a.im) / d, (a.im * r - a.re) / d);
   }
 }
+// 1 / d for d != 0, scaled by a power of two (exact) so |d|^2 cannot over- or
+// underflow; one FP64 division instead of the two of a complex quotient
+__device__ __forceinline__ cx<double> crecip64(cx<double> d) {
+  const double sc = fmax(fabs(d.re), fabs(d.im));
+  const int e = ilogb(sc);
+  const double f = scalbn(1.0, -e);
+  const cx<double> ds = mk(d.re * f, d.im * f);
+  const double r = f / abs2(ds);
+  return mk(ds.re * r, -ds.im * r);
+}
 template <typename To, typename Ti> HD cx<To> ccast(cx<Ti> a) { return mk((To)a.re, (To)a.im); }
 
 // Principal square root.

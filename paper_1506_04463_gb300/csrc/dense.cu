@@ -200,42 +200,13 @@ void launch_broadcast_block(const cxd *X, cxd *Y, size_t count, int copies, cuda
   note_launch();
 }
 
-// ---------------------------------------------------------------------------
-// small products C = op(A) op(B): (m x k) (k x n)
-// ---------------------------------------------------------------------------
-__global__ void k_small_mm(const cxd *A, int opA, const cxd *B, int opB, cxd *C, int m, int k, int n) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * n; e += gridDim.x * blockDim.x) {
-    int i = e / n, j = e - i * n;
-    cxd s = mk(0.0, 0.0);
-    for (int l = 0; l < k; ++l) {
-      cxd a = opA ? conj(A[(size_t)l * m + i]) : A[(size_t)i * k + l];
-      cxd b = opB ? conj(B[(size_t)j * k + l]) : B[(size_t)l * n + j];
-      cfma(s, a, b);
-    }
-    C[e] = s;
-  }
-}
-void small_mm(const cxd *A, int opA, const cxd *B, int opB, cxd *C, int m, int k, int n, cudaStream_t s) {
-  k_small_mm<<<ceil_div(m * n, 128), 128, 0, s>>>(A, opA, B, opB, C, m, k, n);
-  note_launch();
-}
-
 __device__ __forceinline__ double cabs1(cxd a) { return fabs(a.re) + fabs(a.im); }
-// 1 / d for d != 0, scaled by a power of two (exact) so |d|^2 cannot over- or
-// underflow; one FP64 division instead of the two of a complex quotient
-__device__ __forceinline__ cxd crecip(cxd d) {
-  const double sc = fmax(fabs(d.re), fabs(d.im));
-  const int e = ilogb(sc);
-  const double f = scalbn(1.0, -e);
-  const cxd ds = mk(d.re * f, d.im * f);
-  const double r = f / abs2(ds);
-  return mk(ds.re * r, -ds.im * r);
-}
-
 // ---------------------------------------------------------------------------
-// Gauss-Jordan inverse with partial pivoting (one CTA)
+// Gauss-Jordan inverse with partial pivoting (one CTA); nothing to do when
+// *skip (the inverse is already there)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(512) k_small_inv(const cxd *A, int m, cxd *Ainv, cxd *W, int *err) {
+__global__ void __launch_bounds__(512) k_small_inv(const cxd *A, int m, cxd *Ainv, cxd *W, int *err, const int *skip) {
+  if (skip && *skip) return;
   __shared__ cxd f[kMaxM0];
   __shared__ double bv[512];
   __shared__ int bi[512];
@@ -286,7 +257,7 @@ __global__ void __launch_bounds__(512) k_small_inv(const cxd *A, int m, cxd *Ain
     __syncthreads();
     if (tid == 0) {
       const cxd d = W[(size_t)p * m + p];
-      dinv_s = (d.re != 0.0 || d.im != 0.0) ? crecip(d) : mk(0.0, 0.0);
+      dinv_s = (d.re != 0.0 || d.im != 0.0) ? crecip64(d) : mk(0.0, 0.0);
     }
     __syncthreads();
     const cxd dinv = dinv_s;
@@ -305,15 +276,15 @@ __global__ void __launch_bounds__(512) k_small_inv(const cxd *A, int m, cxd *Ain
     __syncthreads();
   }
 }
-void small_inv(const cxd *A, int m, cxd *Ainv, cxd *work, int *d_err, cudaStream_t s) {
-  k_small_inv<<<1, 512, 0, s>>>(A, m, Ainv, work, d_err);
+void small_inv(const cxd *A, int m, cxd *Ainv, cxd *work, int *d_err, const int *skip, cudaStream_t s) {
+  k_small_inv<<<1, 512, 0, s>>>(A, m, Ainv, work, d_err, skip);
   note_launch();
 }
 
 // ---------------------------------------------------------------------------
-// eigendecomposition of a general complex m x m matrix (one CTA)
+// eigendecomposition of a general complex m x m matrix in FP64 (one CTA): the
+// pairs that the refined FP32 decomposition (eig.cu) does not reach
 // ---------------------------------------------------------------------------
-
 
 // work layout: H (m*m; used when H does not fit in shared memory), Z (m*m), E (m*m).
 // H lives in dynamic shared memory (odd row stride) when it fits.  The QR
@@ -357,7 +328,8 @@ __device__ __forceinline__ void givens(cxd a, cxd b, double &c, cxd &s) {
 }
 
 __global__ void __launch_bounds__(256, 1) k_small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *err,
-                                                   int hsm) {
+                                                   int hsm, const int *skip) {
+  if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ cxd v[kMaxM0];
   __shared__ double red[256];
@@ -668,7 +640,7 @@ __global__ void __launch_bounds__(256, 1) k_small_eig(const cxd *A, int m, cxd *
       for (int l2 = j + 1; l2 <= k; ++l2) cfma(s, H[(size_t)j * ld + l2], E[(size_t)l2 * m + k]);
       cxd d = H[(size_t)j * ld + j] - tk;
       if (cabs1(d) < small) d = mk(small, 0.0);
-      E[(size_t)j * m + k] = -(s * crecip(d));
+      E[(size_t)j * m + k] = -(s * crecip64(d));
     }
     lam[k] = tk;
   }
@@ -688,7 +660,7 @@ __global__ void __launch_bounds__(256, 1) k_small_eig(const cxd *A, int m, cxd *
   }
 }
 
-void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *d_err, cudaStream_t s) {
+void small_eig_qr(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *d_err, const int *skip, cudaStream_t s) {
   const size_t hbytes = (size_t)m * (m | 1) * sizeof(cxd);
   const int hsm = hbytes <= 200 * 1024;
   if (hsm) {
@@ -698,7 +670,7 @@ void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *d_err, cud
       attr = true;
     }
   }
-  k_small_eig<<<1, 256, hsm ? hbytes : 0, s>>>(A, m, lam, V, work, d_err, hsm);
+  k_small_eig<<<1, 256, hsm ? hbytes : 0, s>>>(A, m, lam, V, work, d_err, hsm, skip);
   note_launch();
 }
 

@@ -135,6 +135,7 @@ struct feast_nh_ctx {
   bool rr_only = false;       // Rayleigh-Ritz workspace only (one problem of a batch)
   int max_nnz[2] = {0, 0};    // longest row of A and of A^H
   void *fgwork = nullptr;     // FGMRES workspace
+  void *ework = nullptr;      // refined eigendecomposition workspace
   cxf *dfg = nullptr;         // FGMRES correction (node-major, complex float)
   cxd *adiag = nullptr, *bdiag = nullptr;  // diagonals of A and B (Jacobi)
   feast_nh_net *net = nullptr;              // learned preconditioner (not owned)
@@ -617,13 +618,26 @@ int do_rr(feast_nh_ctx *ctx, const cxd *Q, const cxd *Qh, int m, cxd *Y, cxd *Yh
     BQq = ctx->T1;
   }
   proj_gram(ctx, Qh, m, m, BQq, m, m, ctx->BQ);
-  // 3.a  B_Q = V Gamma V^^H ; 2.b spurious ; 3.b-3.c resize and sort
-  small_eig(ctx->BQ, m, ctx->gam, ctx->V, ctx->swork, ctx->d_err, s);
-  if (!cs) small_inv(ctx->V, m, ctx->Vinv, ctx->swork, ctx->d_err, s);
-  launch_gamma_prep(m, ctx->BQ, ctx->gam, ctx->V, ctx->Vinv, ctx->prev_rho, ctx->prev_inside, ctx->have_prev,
-                    ctx->o.mu, ctx->o.eta, cs ? 1 : 0, ctx->S, ctx->Sh, ctx->ord, ctx->d_st, s);
-  check_launch(ctx, "B_Q eigendecomposition");
-  read_status(ctx);
+  // 3.a-3.c: coefficients of U, Uh with Uh^H B U = I, 2.b spurious.  Usually
+  // by elimination (no column can be dropped); otherwise, and for the bilinear
+  // form of a complex symmetric pencil, by B_Q = V Gamma V^^H with the resize
+  // and sort of eq. (resize).
+  bool eig = cs;
+  if (!cs) {
+    CKC(launch_biorth(m, ctx->BQ, ctx->prev_rho, ctx->prev_inside, ctx->have_prev, ctx->o.mu, ctx->o.eta, ctx->S,
+                      ctx->Sh, ctx->d_st, s));
+    read_status(ctx);
+    eig = !ctx->h_st->biorth;
+  }
+  if (eig) {
+    // graded (the filter's values run over many orders), so straight to the FP64 QR
+    small_eig_qr(ctx->BQ, m, ctx->gam, ctx->V, ctx->swork, ctx->d_err, nullptr, s);
+    if (!cs) small_inv(ctx->V, m, ctx->Vinv, ctx->swork, ctx->d_err, nullptr, s);
+    launch_gamma_prep(m, ctx->BQ, ctx->gam, ctx->V, ctx->Vinv, ctx->prev_rho, ctx->prev_inside, ctx->have_prev,
+                      ctx->o.mu, ctx->o.eta, cs ? 1 : 0, ctx->S, ctx->Sh, ctx->ord, ctx->d_st, s);
+    check_launch(ctx, "B_Q eigendecomposition");
+    read_status(ctx);
+  }
   const int mt = ctx->h_st->m_tilde;
   if (mt < 1) {
     ctx->err = "B_Q is zero: the filtered subspace vanished";
@@ -642,15 +656,13 @@ int do_rr(feast_nh_ctx *ctx, const cxd *Q, const cxd *Qh, int m, cxd *Y, cxd *Yh
   }
   proj_gram(ctx, ctx->Uhw, mt, mt, BUu, mt, mt, ctx->BU);
   // 4.b  A_U W = B_U W Lambda via eig(B_U^{-1} A_U); Wh^H = W^{-1} B_U^{-1}
-  small_inv(ctx->BU, mt, ctx->BUinv, ctx->swork, ctx->d_err, s);
-  small_mm(ctx->BUinv, 0, ctx->AU, 0, ctx->Mred, mt, mt, mt, s);
-  small_eig(ctx->Mred, mt, ctx->lam, ctx->W, ctx->swork, ctx->d_err, s);
-  if (cs) {
-    launch_cs_wnorm(mt, ctx->BU, ctx->W, ctx->Wh, s);
-  } else {
-    small_inv(ctx->W, mt, ctx->Winv, ctx->swork, ctx->d_err, s);
-    small_mm(ctx->BUinv, 1, ctx->Winv, 1, ctx->Wh, mt, mt, mt, s);
-  }
+  small_inv_near(ctx->BU, mt, ctx->BUinv, ctx->swork, ctx->ework, ctx->d_err, s);
+  small_prod(mt, ctx->BUinv, ctx->AU, ctx->Mred, 0, s);
+  small_eig(ctx->Mred, mt, ctx->lam, ctx->W, cs ? nullptr : ctx->Winv, ctx->swork, ctx->ework, ctx->d_err, s);
+  if (cs)
+    launch_cs_wnorm(mt, ctx->BU, ctx->W, ctx->Wh, ctx->Winv, s);
+  else
+    small_prod(mt, ctx->Winv, ctx->BUinv, ctx->Wh, 1, s);
   // 4.c  rho_a(lambda)
   launch_rho(mt, ctx->ne, ctx->dz, ctx->dw, ctx->lam, ctx->rho, s);
   // 4.d  Y = U W, Yh = Uh Wh; column scale ||y_i|| = 1
@@ -972,6 +984,7 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     ctx->Winv = dalloc<cxd>(ctx, sm);
     ctx->Wh = dalloc<cxd>(ctx, sm);
     ctx->swork = dalloc<cxd>(ctx, 3 * sm);
+    ctx->ework = dalloc<void>(ctx, small_eig_work_bytes());
     ctx->gchunks = gram_chunks(n);
     ctx->gpart = dalloc<cxd>(ctx, std::max((size_t)ctx->gchunks * sm, gram_tc_part_max(n)));
     ctx->d_fxy = dalloc<int>(ctx, 2 * kMaxM0 * sizeof(int));
@@ -1232,7 +1245,7 @@ feast_nh_status feast_nh_small_eig(feast_nh_ctx *ctx, const void *M, int32_t m, 
   try {
     REQ(M && lambda && V && m >= 1 && m <= kMaxM0, "small_eig: bad arguments (1 <= m <= 128)");
     CKC(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->s));
-    small_eig((const cxd *)M, m, (cxd *)lambda, (cxd *)V, ctx->swork, ctx->d_err, ctx->s);
+    small_eig((const cxd *)M, m, (cxd *)lambda, (cxd *)V, nullptr, ctx->swork, ctx->ework, ctx->d_err, ctx->s);
     check_launch(ctx, "small_eig");
     CKC(cudaMemcpyAsync(ctx->h_small + 1, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
     CKC(cudaStreamSynchronize(ctx->s));

@@ -212,9 +212,17 @@ void launch_broadcast_block(const cxd *X, cxd *Y, size_t count, int copies, cuda
 // *d_err |= bits (host-side fault injection through the device error word).
 void launch_or_bits(int *d_err, int bits, cudaStream_t s);
 
-// Small single-CTA work on m x m matrices in global memory (row-major).
-void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *d_err, cudaStream_t s);
-void small_inv(const cxd *A, int m, cxd *Ainv, cxd *work, int *d_err, cudaStream_t s);
-// C = op(A) * op(B), all m x m (or general k), op: 0 none, 1 conj-transpose.
-void small_mm(const cxd *A, int opA, const cxd *B, int opB, cxd *C, int m, int k, int n, cudaStream_t s);
+// Dense m x m work in global memory (row-major, m <= 128).  small_eig_qr and
+// small_inv run on one CTA and return at once when *skip (may be NULL) is set.
+void small_eig_qr(const cxd *A, int m, cxd *lam, cxd *V, cxd *work, int *d_err, const int *skip, cudaStream_t s);
+void small_inv(const cxd *A, int m, cxd *Ainv, cxd *work, int *d_err, const int *skip, cudaStream_t s);
 
+// ---------------- eig.cu : the same spread over the chip --------------------
+// Eigenvalues, unit eigenvectors V and (if not NULL) V^{-1}; swork: 3 m^2
+// complex, work: small_eig_work_bytes().
+size_t small_eig_work_bytes();
+void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *Vinv, cxd *swork, void *work, int *d_err, cudaStream_t s);
+// Inverse of a matrix that is usually within 1e-3 of the identity.
+void small_inv_near(const cxd *B, int m, cxd *Binv, cxd *swork, void *work, int *d_err, cudaStream_t s);
+// C = A B, or (A B)^H with herm.
+void small_prod(int m, const cxd *A, const cxd *B, cxd *C, int herm, cudaStream_t s);

@@ -78,28 +78,6 @@ __global__ void k_gamma_prep(int m, const cxd *BQ, const cxd *gam, const cxd *V,
   }
 }
 
-// Complex symmetric reduced problem: scale W so that w^T B_U w = 1, Wh = conj(W).
-__global__ void k_cs_wnorm(int m, const cxd *BU, cxd *W, cxd *Wh) {
-  __shared__ cxd t[kMaxM0];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int k = tid; k < m; k += nt) {
-    cxd s = mk(0.0, 0.0);
-    for (int a = 0; a < m; ++a) {
-      cxd bw = mk(0.0, 0.0);
-      for (int b = 0; b < m; ++b) cfma(bw, BU[(size_t)a * m + b], W[(size_t)b * m + k]);
-      cfma(s, W[(size_t)a * m + k], bw);
-    }
-    t[k] = csqrt(s);
-  }
-  __syncthreads();
-  for (int e = tid; e < m * m; e += nt) {
-    const int k = e % m;
-    cxd v = cdiv(W[e], t[k]);
-    W[e] = v;
-    Wh[e] = conj(v);
-  }
-}
-
 // Step 4.c: rho_a(lambda_i) = sum_j w_j / (z_j - lambda_i)   (eq. rational).
 // One warp per eigenvalue, a lane per node: the FP64 quotients (some 50
 // instructions of 64 cycles each) are formed side by side.
@@ -287,10 +265,6 @@ void launch_gamma_prep(int m, const cxd *BQ, const cxd *gam, const cxd *V, const
                        int *ord, RRStatus *st, cudaStream_t s) {
   k_gamma_prep<<<1, 256, 0, s>>>(m, BQ, gam, V, Vinv, prev_rho, prev_inside, have_prev, mu, eta, cs, S, Sh, ord,
                                  st);
-  note_launch();
-}
-void launch_cs_wnorm(int m, const cxd *BU, cxd *W, cxd *Wh, cudaStream_t s) {
-  k_cs_wnorm<<<1, 128, 0, s>>>(m, BU, W, Wh);
   note_launch();
 }
 void launch_rho(int m, int ne, const cxd *z, const cxd *w, const cxd *lam, cxd *rho, cudaStream_t s) {
