@@ -1573,12 +1573,13 @@ void batch_autotune(feast_nh_batch *b) {
   float best = 1e30f;
   int bt = 256, bg = 0, br = 128;
   const int threads_c[] = {256, 512};
-  const int rows_c[] = {64, 256};
+  const int rows_c[] = {16, 64};
+  b->L.side1 = 0;  // one side is enough to compare shapes
   BCK(cudaEventRecord(b->ev[2], b->s));
   for (int th : threads_c) {
     const int occ = batch_fp32(b) ? batch_filter_max_ctas_per_sm<float>(th) : batch_filter_max_ctas_per_sm<double>(th);
     if (occ < 1) continue;
-    for (int per_sm = 1; per_sm <= std::min(occ, 2); per_sm *= 2)
+    for (int per_sm = 1; per_sm <= std::min(occ, 4); per_sm *= 2)
       for (int rows : rows_c) {
         batch_tiles(b, rows);
         b->threads = th;
@@ -1598,6 +1599,7 @@ void batch_autotune(feast_nh_batch *b) {
         }
       }
   }
+  b->L.side1 = 1;
   BCK(cudaEventRecord(b->ev[3], b->s));
   BCK(cudaEventSynchronize(b->ev[3]));
   float tot = 0;
@@ -1714,16 +1716,30 @@ feast_nh_status feast_nh_batch_init(feast_nh_batch **out, int32_t nprob, const f
     b->Qh = balloc<cxd>(b, blk * sizeof(cxd));
     b->X = balloc<cxd>(b, nblk * sizeof(cxd));
     b->diag = balloc<cxd>(b, b->ntot * sizeof(cxd));
-    for (int p = 0; p < nprob; ++p) launch_csr_diag(b->hp[p].A, b->diag + b->hp[p].off, b->s);
+    b->L.kinv = balloc<void>(b, (size_t)ne * b->ntot * (es));
+    for (int p = 0; p < nprob; ++p) {
+      BatchProb &bp = b->hp[p];
+      launch_csr_diag(bp.A, b->diag + bp.off, b->s);
+      const size_t ve = es / (bp.A.cplx ? 1 : 2);  // bytes of a value
+      void *vA = balloc<void>(b, (size_t)bp.A.nnz * ve), *vAH = balloc<void>(b, (size_t)bp.A.nnz * ve);
+      unsigned char *ki = (unsigned char *)b->L.kinv + (size_t)ne * bp.off * es;
+      if (batch_fp32(b))
+        launch_batch_setup<float>(bp.A, bp.AH, b->diag + bp.off, bp.z, ne, (float *)vA, (float *)vAH, (cxf *)ki, b->s);
+      else
+        launch_batch_setup<double>(bp.A, bp.AH, b->diag + bp.off, bp.z, ne, (double *)vA, (double *)vAH, (cxd *)ki,
+                                   b->s);
+      bp.vA = vA;
+      bp.vAH = vAH;
+    }
     for (int k = 0; k < 9; ++k) b->L.kblk[k] = balloc<void>(b, nblk * es);
     // tiles: room for the smallest tile size the tuner tries
     int maxt = 0;
-    for (int p = 0; p < nprob; ++p) maxt += ceil_div(b->hp[p].n, 64);
+    for (int p = 0; p < nprob; ++p) maxt += ceil_div(b->hp[p].n, 16);
     b->max_tiles = maxt;
     b->dtiles = balloc<BatchTile>(b, (size_t)maxt * sizeof(BatchTile));
     b->dprob = balloc<BatchProb>(b, (size_t)nprob * sizeof(BatchProb));
     const size_t PS = (size_t)ne * m0;
-    b->L.part = balloc<void>(b, (size_t)maxt * 2 * PS * es);
+    b->L.part = balloc<void>(b, (size_t)maxt * 4 * PS * es);
     b->L.partd = balloc<double>(b, (size_t)maxt * PS * sizeof(double));
     b->L.partb = balloc<double>(b, (size_t)maxt * m0 * sizeof(double));
     const size_t S = (size_t)nprob * PS;
@@ -1755,7 +1771,6 @@ feast_nh_status feast_nh_batch_init(feast_nh_batch **out, int32_t nprob, const f
     b->L.Yh = b->Yh;
     b->L.Q = b->Q;
     b->L.Qh = b->Qh;
-    b->L.diag = b->diag;
     b->L.X = b->X;
     b->L.tau_min = batch_fp32(b) ? 1e-5 : 0.0;
     // a grid barrier waits at most ~8 s (at 2 GHz) before the launch gives up

@@ -97,6 +97,7 @@ struct BatchProb {
   CsrView A, AH;
   size_t off;
   int n, m, active, tb, te, pad;
+  const void *vA, *vAH;  // values of A, AH in the sweeps' precision (real, or interleaved complex)
   cxd z[kBatchMaxNe], w[kBatchMaxNe];
 };
 struct BatchTile {
@@ -108,7 +109,7 @@ struct BatchScal {
   double *bn2;    // ||Y_c||^2 per (problem, column): nprob * m0
   double *rel;    // relative residual of the last refinement check
   double *stop2;  // Krylov stopping threshold on |r|^2
-  int *act;       // iterating in the current Krylov solve
+  int *act;       // iterating in the current Krylov solve (2: one last update)
   int *act0;      // not yet refined to tolerance
 };
 struct BatchStats {
@@ -123,7 +124,7 @@ struct BatchLaunch {
   const BatchTile *tiles;
   const cxd *Y, *Yh;
   cxd *Q, *Qh;
-  const cxd *diag;
+  const void *kinv; // 1 / (z_j - a_ii), ne x n per problem
   cxd *X;
   void *kblk[9];   // r, rh, p, v, y, s, z, t, d in the Krylov precision
   void *part;
@@ -142,6 +143,10 @@ struct BatchLaunch {
 template <typename T>
 cudaError_t batch_filter_launch(const BatchLaunch &L, int grid, int threads, cudaStream_t s);
 template <typename T> int batch_filter_max_ctas_per_sm(int threads);
+// Values and inverse diagonals of one problem in the sweeps' precision.
+template <typename T>
+void launch_batch_setup(const CsrView &A, const CsrView &AH, const cxd *diag, const cxd *z, int ne, T *vA, T *vAH,
+                        cx<T> *kinv, cudaStream_t s);
 // diag[i] = A_ii (sum of the stored diagonal entries of row i).
 void launch_csr_diag(const CsrView &A, cxd *diag, cudaStream_t s);
 // Deterministic fill of a block with values in [-1, 1] (autotuning input).
