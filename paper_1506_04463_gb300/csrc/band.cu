@@ -908,14 +908,18 @@ __global__ void __launch_bounds__(R *NB / RPT) k_band_solve(int n, int kl, int k
 constexpr int DIB = 16;
 template <typename T>
 __device__ __forceinline__ cx<T> band_ld(const cx<T> *B, size_t o) { return B[o]; }
+// blocks (warps) per CTA: two 16 x 17 tiles each within 48 KB
+template <typename T> struct DiagWarps;
+template <> struct DiagWarps<float> { static constexpr int W = 8; };
+template <> struct DiagWarps<double> { static constexpr int W = 4; };
 template <typename T>
 __global__ void __launch_bounds__(256) k_band_diag_inv(int n, int kl, int ku, const cx<T> *band, size_t ns,
                                                        cx<T> *dinv) {
-  __shared__ cx<T> Lb[8][DIB][DIB + 1];
-  __shared__ cx<T> Ub[8][DIB][DIB + 1];
+  __shared__ cx<T> Lb[DiagWarps<T>::W][DIB][DIB + 1];
+  __shared__ cx<T> Ub[DiagWarps<T>::W][DIB][DIB + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nblk = ceil_div(n, DIB);
-  const int b = blockIdx.x * 8 + warp;
+  const int b = blockIdx.x * DiagWarps<T>::W + warp;
   const int node = blockIdx.y;
   if (b >= nblk) return;
   const int W = kl + ku + 1;
@@ -964,9 +968,11 @@ __global__ void __launch_bounds__(256) k_band_diag_inv(int n, int kl, int ku, co
 template <typename T>
 void launch_band_diag_inv(int n, int kl, int ku, int ne, const cx<T> *band, cx<T> *dinv, cudaStream_t s) {
   const int nblk = ceil_div(n, DIB);
-  k_band_diag_inv<T><<<dim3(ceil_div(nblk, 8), ne), 256, 0, s>>>(n, kl, ku, band, (size_t)n * (kl + ku + 1), dinv);
+  constexpr int wp = DiagWarps<T>::W;
+  k_band_diag_inv<T><<<dim3(ceil_div(nblk, wp), ne), 32 * wp, 0, s>>>(n, kl, ku, band, (size_t)n * (kl + ku + 1), dinv);
   note_launch();
 }
+template void launch_band_diag_inv<double>(int, int, int, int, const cxd *, cxd *, cudaStream_t);
 template void launch_band_diag_inv<float>(int, int, int, int, const cxf *, cxf *, cudaStream_t);
 size_t band_diag_inv_elems(int n, int ne) { return (size_t)ne * ceil_div(n, DIB) * 4 * DIB * DIB; }
 

@@ -92,6 +92,12 @@ struct feast_nh_ctx {
   int klp = 0, kup = 0;     // stored band widths (kl rounded up to even, kl+ku+1 even)
   void *bandT = nullptr;    // FP32: transposed factors for the conjugate-transpose solves
   void *kwork = nullptr;    // BiCGStab workspace
+  // shifted solves by inverted diagonal blocks (blocksolve.cu), of a
+  // tridiagonal pencil (tri.cu), or (neither) by the band's triangular factors
+  bool blk = false, tri = false;
+  void *trico = nullptr;
+  void *blkTc = nullptr, *blkTr = nullptr, *blkys = nullptr;
+  BlockEntries blkE{};
   std::vector<unsigned char> tma;  // tensor maps of band and bandT (empty: no TMA path)
   int nf = 0;              // shifted matrices factorised (ne, or ne/2 with conjugate node pairs)
   std::vector<int> fmap;   // node -> factor slot | conjugate << 16
@@ -180,6 +186,16 @@ P *dalloc(feast_nh_ctx *ctx, size_t bytes) {
   ctx->allocs.push_back(p);
   ctx->pooled.push_back(pooled);
   return reinterpret_cast<P *>(p);
+}
+
+void dfree(feast_nh_ctx *ctx, void *p) {
+  for (size_t i = 0; i < ctx->allocs.size(); ++i)
+    if (ctx->allocs[i] == p) {
+      pool::release(p, ctx->pooled[i], ctx->s);
+      ctx->allocs.erase(ctx->allocs.begin() + i);
+      ctx->pooled.erase(ctx->pooled.begin() + i);
+      return;
+    }
 }
 
 void check_launch(feast_nh_ctx *ctx, const char *what) {
@@ -296,6 +312,38 @@ void fg_precond(void *p, const cxf *v, cxf *z, cudaStream_t s) {
   }
 }
 
+// What the triangular solves need beside the factors: scratch and, in FP32
+// where the TMA form fits, room for the transposed factors, and tensor maps.
+void alloc_lu(feast_nh_ctx *ctx) {
+  const int n = ctx->n;
+  const bool f32 = fp32(ctx);
+  const size_t es = f32 ? sizeof(cxf) : sizeof(cxd);
+  ctx->ysc = dalloc<void>(ctx, es * (f32 ? band_solve_scratch_elems<float>(n, ctx->m0, ctx->ne)
+                                         : band_solve_scratch_elems<double>(n, ctx->m0, ctx->ne)));
+  if (f32 && band_tma_fits(ctx->klp, ctx->kup)) {
+    ctx->bandT = dalloc<void>(ctx, (size_t)ctx->nf * n * (ctx->klp + ctx->kup + 1) * es);
+    ctx->tma.assign(band_tma_bytes(), 0);
+    if (!band_tma_make(ctx->tma.data(), n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band,
+                       (const cxf *)ctx->bandT))
+      ctx->tma.clear();
+  }
+}
+void transpose_lu(feast_nh_ctx *ctx) {
+  if (!ctx->tma.empty())
+    launch_band_transpose(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, (cxf *)ctx->bandT, ctx->s);
+}
+// The explicit inverses (or chunked recurrences) lose too much on this pencil:
+// their memory is given back, and this context keeps to the triangular factors.
+void leave_inverses(feast_nh_ctx *ctx) {
+  for (void **p : {&ctx->trico, &ctx->blkTc, &ctx->blkTr, &ctx->blkys}) {
+    if (*p) dfree(ctx, *p);
+    *p = nullptr;
+  }
+  ctx->blk = ctx->tri = false;
+  alloc_lu(ctx);
+  transpose_lu(ctx);
+}
+
 void factorize(feast_nh_ctx *ctx) {
   if (!banded(ctx)) {
     ctx->factored = true;
@@ -309,12 +357,24 @@ void factorize(feast_nh_ctx *ctx) {
     launch_band_build<float>(ctx->A, Bp, ctx->klp, ctx->kup, ctx->nf, ctx->dzf, (cxf *)ctx->band, ctx->s);
     CKC(band_factor<float>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (cxf *)ctx->band, ctx->d_err, ctx->s));
     launch_band_diag_inv<float>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, (cxf *)ctx->dinv, ctx->s);
-    if (!ctx->tma.empty())
-      launch_band_transpose(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, (cxf *)ctx->bandT, ctx->s);
+    if (ctx->tri)
+      launch_tri_setup<float>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, (cxf *)ctx->trico, ctx->s);
+    else if (ctx->blk)
+      CKC(block_invert<float>(ctx->n, ctx->kl, ctx->ku, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band,
+                              (const cxf *)ctx->dinv, (cxf *)ctx->blkTc, (cxf *)ctx->blkTr, ctx->s));
   } else {
     launch_band_build<double>(ctx->A, Bp, ctx->klp, ctx->kup, ctx->nf, ctx->dzf, (cxd *)ctx->band, ctx->s);
     CKC(band_factor<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (cxd *)ctx->band, ctx->d_err, ctx->s));
+    if (ctx->tri) {
+      launch_tri_setup<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band, (cxd *)ctx->trico, ctx->s);
+    } else if (ctx->blk) {
+      launch_band_diag_inv<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band, (cxd *)ctx->dinv,
+                                   ctx->s);
+      CKC(block_invert<double>(ctx->n, ctx->kl, ctx->ku, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band,
+                               (const cxd *)ctx->dinv, (cxd *)ctx->blkTc, (cxd *)ctx->blkTr, ctx->s));
+    }
   }
+  if (!ctx->blk && !ctx->tri) transpose_lu(ctx);
   CKC(cudaEventRecord(ctx->ev[5], ctx->s));
   if (fp32(ctx))
     launch_band_pivot_stats<float>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, ctx->d_piv, ctx->s);
@@ -442,7 +502,23 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
     const bool f32 = fp32(ctx);
     auto solve = [&](const void *rR, const void *rL, size_t rns, int mode) {
       const int k = ev_begin(ctx, ctx->ev_solve);
-      if (f32)
+      if (ctx->tri && f32)
+        CKC(tri_solve_sides<float>(n, ne, ctx->fmap.data(), (const cxf *)ctx->trico, (const cxf *)rR, (const cxf *)rL,
+                                   rns, m, ctx->Xn, cs ? nullptr : ctx->Xhn, xns, mode, (cxf *)ctx->blkys, ctx->s));
+      else if (ctx->tri)
+        CKC(tri_solve_sides<double>(n, ne, ctx->fmap.data(), (const cxd *)ctx->trico, (const cxd *)rR, (const cxd *)rL,
+                                    rns, m, ctx->Xn, cs ? nullptr : ctx->Xhn, xns, mode, (cxd *)ctx->blkys, ctx->s));
+      else if (ctx->blk && f32)
+        CKC(block_solve_sides<float>(n, ctx->kl, ctx->ku, ne, ctx->fmap.data(), (const cxf *)ctx->blkTc,
+                                     (const cxf *)ctx->blkTr, ctx->blkE, ctx->dz, (const cxf *)rR,
+                                     (const cxf *)rL, rns, m, ctx->Xn, cs ? nullptr : ctx->Xhn, xns, mode,
+                                     (cxf *)ctx->blkys, ctx->d_err, ctx->s));
+      else if (ctx->blk)
+        CKC(block_solve_sides<double>(n, ctx->kl, ctx->ku, ne, ctx->fmap.data(), (const cxd *)ctx->blkTc,
+                                      (const cxd *)ctx->blkTr, ctx->blkE, ctx->dz, (const cxd *)rR,
+                                      (const cxd *)rL, rns, m, ctx->Xn, cs ? nullptr : ctx->Xhn, xns, mode,
+                                      (cxd *)ctx->blkys, ctx->d_err, ctx->s));
+      else if (f32)
         CKC(band_solve_sides<float, float>(n, ctx->klp, ctx->kup, ne, ctx->fmap.data(), (const cxf *)ctx->band,
                                            (const cxf *)ctx->dinv, (const cxf *)rR, (const cxf *)rL, rns, m,
                                            ctx->Xn, cs ? nullptr : ctx->Xhn, xns, mode, (cxf *)ctx->ysc, nullptr,
@@ -453,17 +529,20 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
                                              cs ? nullptr : ctx->Xhn, xns, mode, (cxd *)ctx->ysc, nullptr, ctx->s));
       ev_end(ctx, ctx->ev_solve, k);
     };
-    if (f32) {
-      // the first solve takes the right-hand sides in single precision (the
-      // factors' precision; the refinement restores the rest): they are
-      // staged in the first n x m entries of the residual buffers, which the
-      // first residual overwrites
-      launch_to_cxf(BY, (cxf *)ctx->Rn, (size_t)n * m, ctx->s);
-      if (!cs) launch_to_cxf(BhYh, (cxf *)ctx->Rhn, (size_t)n * m, ctx->s);
-      solve(ctx->Rn, cs ? nullptr : ctx->Rhn, 0, 0);
-    } else {
-      solve(BY, cs ? nullptr : BhYh, 0, 0);
-    }
+    auto first_solve = [&]() {
+      if (f32) {
+        // the first solve takes the right-hand sides in single precision (the
+        // factors' precision; the refinement restores the rest): they are
+        // staged in the first n x m entries of the residual buffers, which the
+        // first residual overwrites
+        launch_to_cxf(BY, (cxf *)ctx->Rn, (size_t)n * m, ctx->s);
+        if (!cs) launch_to_cxf(BhYh, (cxf *)ctx->Rhn, (size_t)n * m, ctx->s);
+        solve(ctx->Rn, cs ? nullptr : ctx->Rhn, 0, 0);
+      } else {
+        solve(BY, cs ? nullptr : BhYh, 0, 0);
+      }
+    };
+    first_solve();
     int g = launch_colnorm2(BY, m, m, n, ctx->colp, ctx->s);
     launch_reduce_parts(ctx->colp, g, m, ctx->bynorm2, ctx->s);
     if (!cs) {
@@ -473,13 +552,16 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
     // The loose first pass of a solve (inner tolerance >= 1e-2, FP32 factors)
     // keeps its single solve unchecked: it only supplies the start subspace of
     // the second iteration, whose refinement verifies the factors; its largest
-    // residual is recorded as NaN ("not measured")
-    const bool unchecked = first_pass && f32;
+    // residual is recorded as NaN ("not measured").  Explicit inverses and
+    // chunked recurrences can lose more than the factors do, so theirs is
+    // measured.
+    const bool unchecked = first_pass && f32 && !ctx->blk && !ctx->tri;
     const int steps = unchecked ? 0 : (ctx->o.inner_max < 1 ? 1 : ctx->o.inner_max);
     if (unchecked) {
       CKC(cudaMemsetAsync(ctx->d_maxrel, 0xFF, sizeof(double), ctx->s));
       ctx->inner_steps = 1;
     }
+    double last = 1.0;  // largest relative residual before the last solve
     for (int it = 0; it < steps; ++it) {
       // residuals only: the node sum Q is formed once, from the final X
       int kr = ev_begin(ctx, ctx->ev_resid);
@@ -504,7 +586,22 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
       CKC(cudaMemcpyAsync(ctx->h_small, ctx->d_maxrel, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
       CKC(cudaStreamSynchronize(ctx->s));
       ctx->inner_steps = it + 1;
-      if (ctx->h_small[0] <= inner_tol) break;
+      const double now = ctx->h_small[0];
+      // FP64 solves by inverted blocks are refined once, which takes them to
+      // the residual of the triangular factors
+      const bool again = ctx->blk && !f32 && it == 0 && steps > 1 && !first_pass;
+      if (now <= inner_tol && !again) break;
+      if ((ctx->blk || ctx->tri) && (!(now <= 0.2 * last) || it + 1 >= steps)) {
+        // too little gained by a step, or none left: the triangular factors
+        // take over, from the start if there is nothing to build on
+        leave_inverses(ctx);
+        if (!(now < 1.0) || it + 1 >= steps) {
+          first_solve();
+          it = -1;
+          continue;
+        }
+      }
+      last = now;
       if (it + 1 < steps) solve(ctx->Rn, cs ? nullptr : ctx->Rhn, xns, 1);
     }
     launch_node_sum(ne, ctx->dw, ctx->Xn, xns, n, m, Q, ctx->s);
@@ -915,18 +1012,47 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     const size_t band_elems = (!banded(ctx) || !inner) ? 0 : (size_t)ctx->nf * n * (ctx->klp + ctx->kup + 1);
     ctx->band = dalloc<void>(ctx, band_elems * es);
     if (krylov(ctx) && inner) ctx->kwork = dalloc<void>(ctx, krylov_work_bytes(n, m0, ne));
-    if (inner && f32 && banded(ctx) && band_tma_fits(ctx->klp, ctx->kup)) {
-      ctx->bandT = dalloc<void>(ctx, band_elems * es);
-      ctx->tma.assign(band_tma_bytes(), 0);
-      if (!band_tma_make(ctx->tma.data(), n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band,
-                         (const cxf *)ctx->bandT))
-        ctx->tma.clear();
+    if (inner && banded(ctx)) {
+      ctx->tri = ctx->kl <= 1 && ctx->ku <= 1;
+      if (ctx->tri) {
+        ctx->trico = dalloc<void>(ctx, tri_elems(n, ctx->nf) * es);
+        ctx->blkys = dalloc<void>(ctx, tri_scratch_elems(n, m0, ne) * es);
+      }
+      if (!ctx->tri && block_solve_fits(ctx->kl, ctx->ku)) {
+        // off-diagonal entries of a row between blocks, both sides
+        int *d_k = dalloc<int>(ctx, sizeof(int)), hk = 0;
+        CKC(cudaMemsetAsync(d_k, 0, sizeof(int), ctx->s));
+        launch_block_count(ctx->A, B ? &ctx->B : nullptr, ctx->kl, ctx->ku, d_k, ctx->s);
+        launch_block_count(ctx->AH, B ? &ctx->BH : nullptr, ctx->kl, ctx->ku, d_k, ctx->s);
+        CKC(cudaMemcpyAsync(&hk, d_k, sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+        CKC(cudaStreamSynchronize(ctx->s));
+        ctx->blk = hk <= kBlockMaxEntries;
+        ctx->blkE.K = hk < 1 ? 1 : hk;
+      }
+      if (!ctx->tri && !ctx->blk) alloc_lu(ctx);
+      if (ctx->blk) {
+        BlockEntries &be = ctx->blkE;
+        const size_t cnt = block_entry_count(n, ctx->kl, ctx->ku, be.K);
+        for (int k = 0; k < 2; ++k) {
+          const CsrView &M = k ? ctx->AH : ctx->A, *N = B ? (k ? &ctx->BH : &ctx->B) : nullptr;
+          be.idx[k] = dalloc<int>(ctx, cnt * sizeof(int));
+          be.va[k] = dalloc<void>(ctx, cnt * es);
+          be.vb[k] = B ? dalloc<void>(ctx, cnt * es) : nullptr;
+          if (f32)
+            launch_block_entries<float>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxf *)be.va[k], (cxf *)be.vb[k],
+                                        ctx->s);
+          else
+            launch_block_entries<double>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxd *)be.va[k], (cxd *)be.vb[k],
+                                         ctx->s);
+        }
+      }
+      if (f32 || ctx->blk) ctx->dinv = dalloc<void>(ctx, band_diag_inv_elems(n, ctx->nf) * es);
+      if (ctx->blk) {
+        ctx->blkTc = dalloc<void>(ctx, block_elems(n, ctx->kl, ctx->ku, ctx->nf) * es);
+        ctx->blkTr = dalloc<void>(ctx, block_elems(n, ctx->kl, ctx->ku, ctx->nf) * es);
+        ctx->blkys = dalloc<void>(ctx, block_scratch_elems(n, ctx->kl, ctx->ku, m0, ne) * es);
+      }
     }
-    const size_t yse = (!banded(ctx) || !inner) ? 0
-                       : f32   ? band_solve_scratch_elems<float>(n, m0, ne)
-                               : band_solve_scratch_elems<double>(n, m0, ne);
-    ctx->ysc = dalloc<void>(ctx, yse * es);
-    if (inner && f32 && banded(ctx)) ctx->dinv = dalloc<void>(ctx, band_diag_inv_elems(n, ctx->nf) * sizeof(cxf));
     if (inner && fgmres(ctx)) {
       ctx->fgwork = dalloc<void>(ctx, fgmres_work_bytes(n, m0, ne, ctx->o.krylov_restart));
       ctx->dfg = dalloc<cxf>(ctx, (size_t)ne * n * m0 * sizeof(cxf));

@@ -43,6 +43,49 @@ void launch_band_pivot_stats(int n, int kl, int ku, int nslots, const cx<T> *ban
 template <typename T> bool band_fits(int kl, int ku);
 template <typename T> bool band_solve_fits(int kl, int ku);
 
+// ---------------- blocksolve.cu : solves with inverted diagonal blocks ------
+// (kl, ku): band of the matrix; (klp, kup): stored band.
+// Off-diagonal entries of A (va) and B (vb, NULL without B) towards the
+// neighbouring blocks, K a row: the matrix [0] and its conjugate transpose [1].
+struct BlockEntries {
+  int K;
+  int *idx[2];
+  void *va[2], *vb[2];
+};
+int block_size(int kl, int ku);
+constexpr int kBlockMaxEntries = 8;  // off-diagonal entries of a row towards a neighbouring block at most
+bool block_solve_fits(int kl, int ku);
+void launch_block_count(const CsrView &A, const CsrView *B, int kl, int ku, int *d_kmax, cudaStream_t s);
+size_t block_entry_count(int n, int kl, int ku, int K);
+template <typename T>
+void launch_block_entries(const CsrView &A, const CsrView *B, int kl, int ku, int K, int *idx, cx<T> *va, cx<T> *vb,
+                          cudaStream_t s);
+size_t block_elems(int n, int kl, int ku, int nf);  // of each copy of the inverses
+size_t block_scratch_elems(int n, int kl, int ku, int m, int ne);
+// Inverses of the diagonal blocks of every factor slot, by columns (Tc) and by
+// rows (Tr), from the factors and the inverses of their 16 x 16 blocks.
+template <typename T>
+cudaError_t block_invert(int n, int kl, int ku, int klp, int kup, int nf, const cx<T> *band, const cx<T> *dinv,
+                         cx<T> *Tc, cx<T> *Tr, cudaStream_t s);
+// As band_solve_sides; d_z: shifts of the nodes.  mode 1 overwrites the
+// right-hand sides.
+template <typename T>
+cudaError_t block_solve_sides(int n, int kl, int ku, int ne, const int *fmap, const cx<T> *Tc, const cx<T> *Tr,
+                              const BlockEntries &en, const cxd *d_z, const cx<T> *rhsR, const cx<T> *rhsL, size_t rns,
+                              int m, cxd *XR, cxd *XL, size_t xns, int mode, cx<T> *ys, int *err, cudaStream_t s);
+
+// ---------------- tri.cu : tridiagonal solves -------------------------------
+struct SolveMap {
+  int f[kMaxNe];  // node -> factor slot | conjugate << 16
+};
+size_t tri_elems(int n, int nf);
+size_t tri_scratch_elems(int n, int m, int ne);
+template <typename T>
+void launch_tri_setup(int n, int klp, int kup, int nf, const cx<T> *band, cx<T> *co, cudaStream_t s);
+template <typename T>
+cudaError_t tri_solve_sides(int n, int ne, const int *fmap, const cx<T> *co, const cx<T> *rhsR, const cx<T> *rhsL,
+                            size_t rns, int m, cxd *XR, cxd *XL, size_t xns, int mode, cx<T> *ys, cudaStream_t s);
+
 // ---------------- spmm.cu : sparse products --------------------------------
 // Q = sum_j w_j X_j over the node-major blocks X; complex128 -> complex64 copy
 void launch_node_sum(int ne, const cxd *d_w, const cxd *X, size_t xns, int n, int m, cxd *Q, cudaStream_t s);
