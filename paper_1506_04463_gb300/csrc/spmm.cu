@@ -9,6 +9,8 @@
 //    A U, B U and the eigen-residuals of eq. (res).
 //  * csr transpose for the conjugate-transpose products A^H, B^H (eq. ql and
 //    the left residual of eq. res).
+#include <algorithm>
+#include <type_traits>
 #include "kernels.h"
 #include "reduce.cuh"
 
@@ -28,23 +30,37 @@ __device__ __forceinline__ void csr_fma(cxd &acc, const CsrView &M, int64_t k, c
 // ---------------------------------------------------------------------------
 // multi-shift residual + node accumulation
 // ---------------------------------------------------------------------------
+// Bound by the FP64 pipe, which a warp instruction takes for 64 cycles whatever
+// the lanes it serves, so FP64 instructions are what counts: without B the
+// diagonal entries of A are folded into the shifts (z_j - a_ii, once a row and
+// node instead of once a column), the squares go into their sum as two FMAs,
+// and Q is formed for eight rows at a time with full warps.  The rows' other
+// entries are staged, so that the gathers of a row are issued together; four
+// CTAs an SM, since fewer registers spill.  n = 44521, 15 nodes, 45 columns,
+// 5 entries a row, with Q: 1348 -> 989 us; n = 90000, 16 nodes, 62 columns,
+// FP32 residual without Q: 2.95 -> 2.66 ms (bound by the conversions to and
+// from FP32 and 12 FMAs, 2.5 ms).
 constexpr int kMsThreads = 256;
 constexpr int kMsMaxPairs = 8;  // ne*m <= 2048
+constexpr int kMsRows = 8;      // rows between two barriers
+constexpr int kMsStage = 160;   // entries of A they may have to be staged
 
-template <typename Tout, bool ACPLX, bool BCPLX>
-__global__ void __launch_bounds__(kMsThreads)
-    k_multishift_residual(CsrView A, CsrView B, int hasB, int ne, const cxd *__restrict__ z,
+template <typename Tout, bool ACPLX, bool BCPLX, bool HASB>
+__global__ void __launch_bounds__(kMsThreads, 4)
+    k_multishift_residual(CsrView A, CsrView B, int ne, const cxd *__restrict__ z,
                           const cxd *__restrict__ w, const cxd *__restrict__ X, size_t xns,
                           const cxd *__restrict__ BY, cx<Tout> *__restrict__ R, cxd *__restrict__ Q,
                           double *__restrict__ partial, int m, int rows_per_cta, const int *skip) {
   if (skip && *skip) return;
-  __shared__ cxd zs[kMaxNe], ws[kMaxNe];
+  using Val = typename std::conditional<ACPLX, cxd, double>::type;
+  __shared__ cxd ws[kMaxNe], zs[HASB ? 1 : kMsRows][kMaxNe];
+  __shared__ Val sval[kMsStage];
+  __shared__ int scol[kMsStage], sbeg[kMsRows], send[kMsRows];
   const int tid = threadIdx.x;
   if (tid < ne) {
-    zs[tid] = z[tid];
     ws[tid] = w[tid];
+    if (HASB) zs[0][tid] = z[tid];
   }
-  __syncthreads();
   const int P = ne * m;
   const int n = A.n;
   const int rbeg = blockIdx.x * rows_per_cta;
@@ -53,36 +69,87 @@ __global__ void __launch_bounds__(kMsThreads)
 #pragma unroll
   for (int q = 0; q < kMsMaxPairs; ++q) nacc[q] = 0.0;
 
-  for (int i = rbeg; i < rend; ++i) {
-    const int64_t ka = A.rowptr[i], kae = A.rowptr[i + 1];
+  for (int i0 = rbeg; i0 < rend; i0 += kMsRows) {
+    const int rows = min(kMsRows, rend - i0);
+    const int64_t k0 = A.rowptr[i0];
+    const bool staged = A.rowptr[i0 + rows] - k0 <= kMsStage;
+    __syncthreads();
+    if (!HASB) {
+      // z_j - a_ii of the chunk's rows (entries of one position add up)
+      for (int e = tid; e < rows * ne; e += kMsThreads) {
+        const int r = e / ne, j = e - r * ne, i = i0 + r;
+        cxd d = z[j];
+        for (int64_t k = A.rowptr[i]; k < A.rowptr[i + 1]; ++k)
+          if (A.colind[k] == i) d = d - csr_val(A, k);
+        zs[r][j] = d;
+      }
+    }
+    if (staged && tid < 32 * rows && (tid & 31) == 0) {
+      const int r = tid >> 5, i = i0 + r;
+      int o = (int)(A.rowptr[i] - k0);
+      sbeg[r] = o;
+      for (int64_t k = A.rowptr[i]; k < A.rowptr[i + 1]; ++k) {
+        const int col = A.colind[k];
+        if (!HASB && col == i) continue;
+        scol[o] = col;
+        if constexpr (ACPLX) sval[o] = csr_val(A, k); else sval[o] = A.val[k];
+        ++o;
+      }
+      send[r] = o;
+    }
+    __syncthreads();
+    for (int r = 0; r < rows; ++r) {
+      const int i = i0 + r;
 #pragma unroll
-    for (int q = 0; q < kMsMaxPairs; ++q) {
-      const int pair = tid + kMsThreads * q;
-      if (pair < P) {
-        const int j = pair / m, c = pair - j * m;
-        const cxd *Xj = X + (size_t)j * xns;
-        cxd acc = BY ? BY[(size_t)i * m + c] : mk(0.0, 0.0);
-        cxd bx;
-        if (hasB) {
-          bx = mk(0.0, 0.0);
-          for (int64_t k = B.rowptr[i]; k < B.rowptr[i + 1]; ++k)
-            csr_fma<BCPLX>(bx, B, k, Xj[(size_t)B.colind[k] * m + c]);
-        } else {
-          bx = Xj[(size_t)i * m + c];
+      for (int q = 0; q < kMsMaxPairs; ++q) {
+        const int pair = tid + kMsThreads * q;
+        if (pair < P) {
+          const int j = pair / m, c = pair - j * m;
+          const cxd *Xj = X + (size_t)j * xns + c;
+          cxd acc = BY ? BY[(size_t)i * m + c] : mk(0.0, 0.0);
+          if (HASB) {
+            cxd bx = mk(0.0, 0.0);
+            for (int64_t k = B.rowptr[i]; k < B.rowptr[i + 1]; ++k)
+              csr_fma<BCPLX>(bx, B, k, Xj[(size_t)B.colind[k] * m]);
+            cfms(acc, zs[0][j], bx);
+          } else {
+            cfms(acc, zs[r][j], Xj[(size_t)i * m]);
+          }
+          if (staged) {
+            const int ke = send[r];
+#pragma unroll 4
+            for (int k = sbeg[r]; k < ke; ++k) {
+              const cxd x = Xj[(size_t)scol[k] * m];
+              if constexpr (ACPLX) {
+                cfma(acc, sval[k], x);
+              } else {
+                acc.re = fma(sval[k], x.re, acc.re);
+                acc.im = fma(sval[k], x.im, acc.im);
+              }
+            }
+          } else {
+            for (int64_t k = A.rowptr[i]; k < A.rowptr[i + 1]; ++k) {
+              const int col = A.colind[k];
+              if (HASB || col != i) csr_fma<ACPLX>(acc, A, k, Xj[(size_t)col * m]);
+            }
+          }
+          const cx<Tout> ro = ccast<Tout>(acc);
+          if (R) R[(size_t)j * xns + (size_t)i * m + c] = ro;
+          // the norm of the stored residual, squared in its own precision
+          if constexpr (sizeof(Tout) == 8)
+            nacc[q] = fma(ro.re, ro.re, fma(ro.im, ro.im, nacc[q]));
+          else
+            nacc[q] += (double)(ro.re * ro.re + ro.im * ro.im);
         }
-        cfms(acc, zs[j], bx);
-        for (int64_t k = ka; k < kae; ++k) csr_fma<ACPLX>(acc, A, k, Xj[(size_t)A.colind[k] * m + c]);
-        const cx<Tout> ro = ccast<Tout>(acc);
-        if (R) R[(size_t)j * xns + (size_t)i * m + c] = ro;
-        // the norm of the stored residual, squared in its own precision
-        nacc[q] += (double)(ro.re * ro.re + ro.im * ro.im);
       }
     }
     if (Q) {
-      for (int c = tid; c < m; c += kMsThreads) {
+      for (int e = tid; e < rows * m; e += kMsThreads) {
+        const size_t o = (size_t)i0 * m + e;
         cxd qv = mk(0.0, 0.0);
-        for (int j = 0; j < ne; ++j) cfma(qv, ws[j], X[(size_t)j * xns + (size_t)i * m + c]);
-        Q[(size_t)i * m + c] = qv;
+#pragma unroll 4
+        for (int j = 0; j < ne; ++j) cfma(qv, ws[j], X[(size_t)j * xns + o]);
+        Q[o] = qv;
       }
     }
   }
@@ -136,6 +203,20 @@ static int ms_grid(int n) {
   return g < 1 ? 1 : g;
 }
 
+#define MS_LAUNCH(AC, BC, HB, SKIP)                                                                         \
+  k_multishift_residual<Tout, AC, BC, HB><<<g, kMsThreads, 0, s>>>(A, Bv, ne, d_z, d_w, X, xns, BY, R, Q, \
+                                                                   partial, m, rpc, SKIP)
+#define MS_CALL(SKIP)                                                                                       \
+  do {                                                                                                      \
+    if (!B) {                                                                                               \
+      if (A.cplx) MS_LAUNCH(true, false, false, SKIP); else MS_LAUNCH(false, false, false, SKIP);           \
+    } else if (A.cplx) {                                                                                    \
+      if (bc) MS_LAUNCH(true, true, true, SKIP); else MS_LAUNCH(true, false, true, SKIP);                   \
+    } else {                                                                                                \
+      if (bc) MS_LAUNCH(false, true, true, SKIP); else MS_LAUNCH(false, false, true, SKIP);                 \
+    }                                                                                                       \
+  } while (0)
+
 template <typename Tout>
 int launch_multishift_residual(const CsrView &A, const CsrView *B, int ne, const cxd *d_z, const cxd *d_w,
                                const cxd *X, const cxd *BY, cx<Tout> *R, cxd *Q, double *partial, int m,
@@ -146,16 +227,8 @@ int launch_multishift_residual(const CsrView &A, const CsrView *B, int ne, const
   const size_t xns = (size_t)A.n * m;
   CsrView Bv = B ? *B : A;
   const bool bc = B ? B->cplx : false;
-#define MS_LAUNCH(AC, BC)                                                                                \
-  k_multishift_residual<Tout, AC, BC><<<g, kMsThreads, 0, s>>>(A, Bv, B != nullptr, ne, d_z, d_w, X, xns, \
-                                                               BY, R, Q, partial, m, rpc, d_skip)
-  if (A.cplx) {
-    if (bc) MS_LAUNCH(true, true); else MS_LAUNCH(true, false);
-  } else {
-    if (bc) MS_LAUNCH(false, true); else MS_LAUNCH(false, false);
-  }
+  MS_CALL(d_skip);
   note_launch();
-#undef MS_LAUNCH
   return g;
 }
 template int launch_multishift_residual<double>(const CsrView &, const CsrView *, int, const cxd *, const cxd *,
@@ -182,21 +255,15 @@ int launch_multishift_residual_capped(const CsrView &A, const CsrView *B, int ne
   const size_t xns = (size_t)A.n * m;
   CsrView Bv = B ? *B : A;
   const bool bc = B ? B->cplx : false;
-#define MS_LAUNCH(AC, BC)                                                                                \
-  k_multishift_residual<Tout, AC, BC><<<g, kMsThreads, 0, s>>>(A, Bv, B != nullptr, ne, d_z, d_w, X, xns, \
-                                                               BY, R, Q, partial, m, rpc, nullptr)
-  if (A.cplx) {
-    if (bc) MS_LAUNCH(true, true); else MS_LAUNCH(true, false);
-  } else {
-    if (bc) MS_LAUNCH(false, true); else MS_LAUNCH(false, false);
-  }
-#undef MS_LAUNCH
+  MS_CALL(nullptr);
   note_launch();
   return g;
 }
 template int launch_multishift_residual_capped<double>(const CsrView &, const CsrView *, int, const cxd *,
                                                        const cxd *, const cxd *, const cxd *, cxd *, cxd *, double *,
                                                        int, int, cudaStream_t);
+#undef MS_CALL
+#undef MS_LAUNCH
 
 // One CTA per 4 (node, column) pairs, 64 threads a pair: at 1216 partials and
 // 2048 pairs this took 179 us with a thread per pair (a chain of 1216 loads);
