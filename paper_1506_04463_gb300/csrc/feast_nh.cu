@@ -139,7 +139,6 @@ struct feast_nh_ctx {
   double piv_min = 0, piv_max = 0;
   unsigned inject_bits = 0;   // host-requested device error bits (testing aid)
   bool rr_only = false;       // Rayleigh-Ritz workspace only (one problem of a batch)
-  int max_nnz[2] = {0, 0};    // longest row of A and of A^H
   void *fgwork = nullptr;     // FGMRES workspace
   void *ework = nullptr;      // refined eigendecomposition workspace
   cxf *dfg = nullptr;         // FGMRES correction (node-major, complex float)
@@ -289,11 +288,11 @@ void fg_apply(void *p, const cxf *x, cxf *y, cudaStream_t s) {
   const FgSide *f = static_cast<const FgSide *>(p);
   feast_nh_ctx *ctx = f->ctx;
   if (f->side == 0)
-    launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->ne, ctx->dz, 0, x, y, f->m, 0,
-                               ctx->max_nnz[0], s);
+    launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 0, x, y,
+                               f->m, s);
   else
-    launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->ne, ctx->dz, 1, x, y, f->m, 0,
-                               ctx->max_nnz[1], s);
+    launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 1, x, y,
+                               f->m, s);
 }
 void fg_precond(void *p, const cxf *v, cxf *z, cudaStream_t s) {
   const FgSide *f = static_cast<const FgSide *>(p);
@@ -955,14 +954,6 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     REQ(ext[2] == 0, "malformed CSR: a row pointer or a column index of A or B is out of range");
     ctx->AH = transpose_view(ctx, ctx->A);
     if (B) ctx->BH = transpose_view(ctx, ctx->B);
-    {
-      int *d_mx = dalloc<int>(ctx, 2 * sizeof(int));
-      CKC(cudaMemsetAsync(d_mx, 0, 2 * sizeof(int), ctx->s));
-      launch_max_row_nnz(ctx->A, d_mx, ctx->s);
-      launch_max_row_nnz(ctx->AH, d_mx + 1, ctx->s);
-      CKC(cudaMemcpyAsync(ctx->max_nnz, d_mx, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
-      CKC(cudaStreamSynchronize(ctx->s));
-    }
     ctx->kl = ext[0];
     ctx->ku = ext[1];
     // stored band: kl rounded up to even and kl+ku+1 even, so that band rows and
@@ -1354,11 +1345,11 @@ feast_nh_status feast_nh_multishift_spmm(feast_nh_ctx *ctx, const void *P, void 
     REQ(P && V && m >= 1 && m <= ctx->m0 && (side == 0 || side == 1), "multishift_spmm: bad arguments");
     REQ(!ctx->rr_only, "multishift_spmm: context has no operator");
     if (side == 0)
-      launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->ne, ctx->dz, 0, (const cxf *)P,
-                                 (cxf *)V, m, 0, ctx->max_nnz[0], ctx->s);
+      launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 0,
+                                 (const cxf *)P, (cxf *)V, m, ctx->s);
     else
-      launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->ne, ctx->dz, 1, (const cxf *)P,
-                                 (cxf *)V, m, 0, ctx->max_nnz[1], ctx->s);
+      launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 1,
+                                 (const cxf *)P, (cxf *)V, m, ctx->s);
     check_launch(ctx, "multishift_spmm");
   } catch (const Fail &f) {
     return f.st;

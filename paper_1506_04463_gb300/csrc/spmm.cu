@@ -494,182 +494,233 @@ cudaError_t csr_transpose(const CsrView &A, int32_t *rowptr_t, int32_t *colind_t
 
 // ---------------------------------------------------------------------------
 // FP32 multi-shift operator of the Krylov sweeps: V_j = (z_j B - A) P_j for
-// every node j and column c in one pass over A and B (left side: the
-// conjugate-transpose CSR with conj(z_j)).  P, V: node-major ne blocks of
-// n x m complex float, row-major.  One warp per (node, row) task, tasks
-// node-major so that the warps in flight sweep neighbouring rows of one node
-// (stencil neighbours are read from L2); a lane holds VW consecutive columns
-// (VW = 2: one 16-byte load per gathered row), the CSR row is read by all
-// lanes at the same address (broadcast).
+// every node j and column c (left side: the conjugate-transpose CSR with
+// conj(z_j)).  P, V: node-major ne blocks of n x m complex float, row-major.
+// Bound by the gathers of P's rows out of L2.  G lanes a row, two columns a
+// lane (one 16-byte load per gathered row where m is even), so that narrow
+// blocks fill their warps with several rows.  A lane loads and converts one
+// entry of the row, which the group's lanes then read by shuffles: converting
+// in every lane took the FP64 pipe 64 cycles a warp and entry.
+// The rows are walked for ng nodes at a time, as many as keep what the rows in
+// flight reach (their number plus the band's width) within kGatherBytes, a
+// third of L2.  Rows of up to U entries keep them in registers for all nodes.
+// 8 nodes of 50021 rows, 9 random entries each, 48 columns of P (154 MB):
+// 203 us with all nodes at once and a warp a row, 185 without the registers,
+// 149 us (the gathers are 1.5 GB, 10 TB/s out of L2); its transpose, with rows
+// of up to 25 entries, 352 -> 248 us; 200000 rows, 16 columns 654 -> 330; the
+// 300 x 300 grid, 16 columns 124 -> 51, 48 columns 144 -> 154.
 // ---------------------------------------------------------------------------
-template <int VW> struct VecF;
-template <> struct VecF<1> { using T = float2; };
-template <> struct VecF<2> { using T = float4; };
-
-template <bool CPLX>
-__device__ __forceinline__ cxf csr_valf(const CsrView &M, int64_t k) {
-  if (CPLX) {
-    const cxd v = reinterpret_cast<const cxd *>(M.val)[k];
-    return mk((float)v.re, M.conj_vals ? -(float)v.im : (float)v.im);
-  }
-  return mk((float)M.val[k], 0.f);
+// Two columns a lane: neighbours (PAIR, rows start on 16 bytes), or G apart
+// where m is odd.
+template <bool PAIR, int G> __device__ __forceinline__ float4 load2(const cxf *p, bool second) {
+  if constexpr (PAIR) return *reinterpret_cast<const float4 *>(p);
+  const float2 a = *reinterpret_cast<const float2 *>(p);
+  float2 b = make_float2(0.f, 0.f);
+  if (second) b = *reinterpret_cast<const float2 *>(p + G);
+  return make_float4(a.x, a.y, b.x, b.y);
 }
-
-template <int VW>
-__device__ __forceinline__ void vfms(typename VecF<VW>::T &acc, cxf a, const typename VecF<VW>::T &x) {
-  // acc -= a * x (VW complex lanes)
-  acc.x = fmaf(-a.re, x.x, acc.x);
-  acc.x = fmaf(a.im, x.y, acc.x);
-  acc.y = fmaf(-a.re, x.y, acc.y);
-  acc.y = fmaf(-a.im, x.x, acc.y);
-  if constexpr (VW == 2) {
-    acc.z = fmaf(-a.re, x.z, acc.z);
-    acc.z = fmaf(a.im, x.w, acc.z);
-    acc.w = fmaf(-a.re, x.w, acc.w);
-    acc.w = fmaf(-a.im, x.z, acc.w);
+template <bool PAIR, int G> __device__ __forceinline__ void store2(cxf *p, float4 v, bool second) {
+  if constexpr (PAIR) {
+    *reinterpret_cast<float4 *>(p) = v;
+  } else {
+    *reinterpret_cast<float2 *>(p) = make_float2(v.x, v.y);
+    if (second) *reinterpret_cast<float2 *>(p + G) = make_float2(v.z, v.w);
   }
 }
-template <int VW>
-__device__ __forceinline__ void vfma(typename VecF<VW>::T &acc, cxf a, const typename VecF<VW>::T &x) {
+
+// acc += a * x (two complex lanes)
+template <bool CPLX> __device__ __forceinline__ void vfma(float4 &acc, cxf a, const float4 &x) {
   acc.x = fmaf(a.re, x.x, acc.x);
-  acc.x = fmaf(-a.im, x.y, acc.x);
   acc.y = fmaf(a.re, x.y, acc.y);
-  acc.y = fmaf(a.im, x.x, acc.y);
-  if constexpr (VW == 2) {
-    acc.z = fmaf(a.re, x.z, acc.z);
+  acc.z = fmaf(a.re, x.z, acc.z);
+  acc.w = fmaf(a.re, x.w, acc.w);
+  if constexpr (CPLX) {
+    acc.x = fmaf(-a.im, x.y, acc.x);
+    acc.y = fmaf(a.im, x.x, acc.y);
     acc.z = fmaf(-a.im, x.w, acc.z);
-    acc.w = fmaf(a.re, x.w, acc.w);
     acc.w = fmaf(a.im, x.z, acc.w);
   }
 }
 
-// One warp per row i, all nodes: the row's CSR entries (up to KMAX) are
-// loaded once into registers and reused for every node j; the gathers of one
-// node (one 16-byte load per lane and entry) are independent, so a lane has
-// up to KMAX + 1 loads in flight per node.  Rows longer than KMAX, and a
-// non-identity B, take the general loop.
-template <bool ACPLX, bool BCPLX, bool HASB, int VW, int KMAX>
-__global__ void __launch_bounds__(256) k_multishift_spmm_f32(CsrView A, CsrView B, int ne, const cxd *__restrict__ z,
-                                                             int conj_z, const cxf *__restrict__ P,
-                                                             cxf *__restrict__ V, int n, int m) {
-  using V4 = typename VecF<VW>::T;
+// A row's entries in the lanes of its group, G at a time
+template <bool CPLX, int G> struct RowPart {
+  int col;
+  cxf val;
+  __device__ __forceinline__ void load(const CsrView &M, int64_t beg, int cnt, int base, float sign) {
+    const int k = base + (threadIdx.x & (G - 1));
+    col = 0;
+    val = mk(0.f, 0.f);
+    if (k < cnt) {
+      col = M.colind[beg + k];
+      if constexpr (CPLX) {
+        const cxd v = reinterpret_cast<const cxd *>(M.val)[beg + k];
+        val = mk(sign * (float)v.re, (M.conj_vals ? -sign : sign) * (float)v.im);
+      } else {
+        val = mk(sign * (float)M.val[beg + k], 0.f);
+      }
+    }
+  }
+  // acc += the product of entries base .. of a row of cnt (most: of the warp's
+  // rows), the gathers of U entries issued together
+  template <int U, bool PAIR>
+  __device__ __forceinline__ void apply(float4 &acc, int base, int cnt, int most, const cxf *Pc, int m,
+                                        bool ok, bool second) const {
+    const int nb = min(G, most - base), left = ok ? min(G, cnt - base) : 0;
+    for (int k = 0; k < nb; k += U) {
+      float4 x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int cu = __shfl_sync(0xffffffffu, col, k + u, G);
+        x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k + u < left) x[u] = load2<PAIR, G>(Pc + (size_t)cu * m, second);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        cxf v;
+        v.re = __shfl_sync(0xffffffffu, val.re, k + u, G);
+        v.im = CPLX ? __shfl_sync(0xffffffffu, val.im, k + u, G) : 0.f;
+        if (k + u < left) vfma<CPLX>(acc, v, x[u]);
+      }
+    }
+  }
+};
+
+constexpr int kSpThreads = 256;
+template <bool ACPLX, bool BCPLX, bool HASB, bool PAIR, int G, int U>
+__global__ void __launch_bounds__(kSpThreads, U == 5 ? 4 : PAIR ? 3 : 2)
+    k_multishift_spmm_f32(CsrView A, CsrView B, int ne, const cxd *__restrict__ z, int conj_z,
+                          const cxf *__restrict__ P, cxf *__restrict__ V, int n, int m, int ng) {
   __shared__ cxf zs[kMaxNe];
   if (threadIdx.x < ne) {
     const cxd zz = z[threadIdx.x];
     zs[threadIdx.x] = mk((float)zz.re, conj_z ? -(float)zz.im : (float)zz.im);
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int warp = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nwarps = (int)(((long long)gridDim.x * blockDim.x) >> 5);
+  constexpr int RPW = 32 / G, kShort = U < G ? U : G;
+  const int lane = threadIdx.x & 31, gl = lane & (G - 1);
+  const int warp = (int)(((long long)blockIdx.x * kSpThreads + threadIdx.x) >> 5);
+  const int nwarps = (int)(((long long)gridDim.x * kSpThreads) >> 5);
   const size_t xns = (size_t)n * m;
-  for (int i = warp; i < n; i += nwarps) {
-    const int64_t ka = A.rowptr[i];
-    const int nk = (int)(A.rowptr[i + 1] - ka);
-    int col[KMAX];
-    cxf av[KMAX];
+  for (int j0 = 0; j0 < ne; j0 += ng) {
+    const int j1 = min(ne, j0 + ng);
+    for (int ib = warp * RPW; ib < n; ib += nwarps * RPW) {
+      const int i = ib + lane / G;
+      const bool row = i < n;
+      const int64_t ka = row ? A.rowptr[i] : 0, kb = HASB && row ? B.rowptr[i] : 0;
+      const int na = row ? (int)(A.rowptr[i + 1] - ka) : 0, nb = HASB && row ? (int)(B.rowptr[i + 1] - kb) : 0;
+      const int ma = __reduce_max_sync(0xffffffffu, na), mb = HASB ? __reduce_max_sync(0xffffffffu, nb) : 0;
+      RowPart<ACPLX, G> ra;  // -A
+      RowPart<BCPLX, G> rb;
+      ra.load(A, ka, na, 0, -1.f);
+      if (HASB) rb.load(B, kb, nb, 0, 1.f);
+      for (int c0 = 0; c0 < m; c0 += 2 * G) {
+        const int c = c0 + (PAIR ? 2 * gl : gl);
+        const bool ok = row && c < m, second = !PAIR && c + G < m;
+        if (!HASB && ma <= kShort) {
+          // short rows, the usual case: their entries in registers for all nodes
+          int col[kShort];
+          cxf v[kShort];
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-      col[k] = k < nk ? A.colind[ka + k] : i;
-      av[k] = k < nk ? csr_valf<ACPLX>(A, ka + k) : mk(0.f, 0.f);
-    }
-    const bool fast = !HASB && nk <= KMAX;
-    for (int c = lane * VW; c < m; c += 32 * VW) {
-#pragma unroll 2
-      for (int j = 0; j < ne; ++j) {
-        const cxf *Pj = P + (size_t)j * xns;
-        V4 acc;
-        acc.x = acc.y = 0.f;
-        if constexpr (VW == 2) acc.z = acc.w = 0.f;
-        if (fast) {
-          V4 xs[KMAX];
-#pragma unroll
-          for (int k = 0; k < KMAX; ++k) xs[k] = *reinterpret_cast<const V4 *>(Pj + (size_t)col[k] * m + c);
-          vfma<VW>(acc, zs[j], *reinterpret_cast<const V4 *>(Pj + (size_t)i * m + c));
-#pragma unroll
-          for (int k = 0; k < KMAX; ++k) vfms<VW>(acc, av[k], xs[k]);
-        } else {
-          if (HASB) {
-            V4 bx;
-            bx.x = bx.y = 0.f;
-            if constexpr (VW == 2) bx.z = bx.w = 0.f;
-            for (int64_t k = B.rowptr[i]; k < B.rowptr[i + 1]; ++k)
-              vfma<VW>(bx, csr_valf<BCPLX>(B, k), *reinterpret_cast<const V4 *>(Pj + (size_t)B.colind[k] * m + c));
-            vfma<VW>(acc, zs[j], bx);
-          } else {
-            vfma<VW>(acc, zs[j], *reinterpret_cast<const V4 *>(Pj + (size_t)i * m + c));
+          for (int u = 0; u < kShort; ++u) {
+            col[u] = __shfl_sync(0xffffffffu, ra.col, u, G);
+            if (u >= na) col[u] = i;  // value zero
+            v[u].re = __shfl_sync(0xffffffffu, ra.val.re, u, G);
+            v[u].im = ACPLX ? __shfl_sync(0xffffffffu, ra.val.im, u, G) : 0.f;
           }
-          for (int k = 0; k < nk; ++k)
-            vfms<VW>(acc, csr_valf<ACPLX>(A, ka + k), *reinterpret_cast<const V4 *>(Pj + (size_t)A.colind[ka + k] * m + c));
+          if (!ok) continue;
+#pragma unroll 2
+          for (int j = j0; j < j1; ++j) {
+            const cxf *Pc = P + (size_t)j * xns + c;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), x[kShort];
+            const float4 own = load2<PAIR, G>(Pc + (size_t)i * m, second);
+#pragma unroll
+            for (int u = 0; u < kShort; ++u) {
+              x[u] = load2<PAIR, G>(Pc + (size_t)col[u] * m, second);
+            }
+#pragma unroll
+            for (int u = 0; u < kShort; ++u) vfma<ACPLX>(acc, v[u], x[u]);
+            vfma<true>(acc, zs[j], own);
+            store2<PAIR, G>(V + (size_t)j * xns + (size_t)i * m + c, acc, second);
+          }
+          continue;
         }
-        *reinterpret_cast<V4 *>(V + (size_t)j * xns + (size_t)i * m + c) = acc;
+        for (int j = j0; j < j1; ++j) {
+          const cxf *Pc = P + (size_t)j * xns + c;
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), bx = acc;
+          if (HASB) {
+            rb.template apply<U, PAIR>(bx, 0, nb, mb, Pc, m, ok, second);
+            for (int base = G; base < mb; base += G) {
+              RowPart<BCPLX, G> more;
+              more.load(B, kb, nb, base, 1.f);
+              more.template apply<U, PAIR>(bx, base, nb, mb, Pc, m, ok, second);
+            }
+          } else if (ok) {
+            bx = load2<PAIR, G>(Pc + (size_t)i * m, second);
+          }
+          ra.template apply<U, PAIR>(acc, 0, na, ma, Pc, m, ok, second);
+          for (int base = G; base < ma; base += G) {
+            RowPart<ACPLX, G> more;
+            more.load(A, ka, na, base, -1.f);
+            more.template apply<U, PAIR>(acc, base, na, ma, Pc, m, ok, second);
+          }
+          vfma<true>(acc, zs[j], bx);
+          if (ok) store2<PAIR, G>(V + (size_t)j * xns + (size_t)i * m + c, acc, second);
+        }
       }
     }
   }
 }
 
-// Longest row of a CSR matrix (entries), for the register row length of the
-// FP32 operator.
-__global__ void k_max_row_nnz(CsrView A, int *out) {
-  int mx = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x)
-    mx = max(mx, (int)(A.rowptr[i + 1] - A.rowptr[i]));
-  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
-}
-void launch_max_row_nnz(const CsrView &A, int *d_out, cudaStream_t s) {
-  k_max_row_nnz<<<min(1024, ceil_div(A.n, 256)), 256, 0, s>>>(A, d_out);
-  note_launch();
-}
 
-template <int KMAX>
-static long long spmm_f32_dispatch(const CsrView &A, const CsrView *B, int ne, const cxd *d_z, int conj_z,
-                                   const cxf *P, cxf *V, int m, int grid_per_sm, cudaStream_t s) {
+constexpr size_t kGatherBytes = 40u << 20;
+
+template <bool PAIR, int G>
+static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z, const cxf *P,
+                           cxf *V, int m, cudaStream_t s) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  CsrView Bv = B ? *B : A;
-  const bool bc = B ? B->cplx : false;
-  const bool vec2 = (m % 2) == 0;
-  long long g = 0;
-#define SPF(AC, BC, HB, VW)                                                                                 \
-  do {                                                                                                      \
-    auto kern = k_multishift_spmm_f32<AC, BC, HB, VW, KMAX>;                                                \
-    int occ = 0;                                                                                            \
-    if (grid_per_sm > 0) occ = grid_per_sm;                                                                 \
-    else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, 0) != cudaSuccess || occ < 1) \
-      occ = 1;                                                                                              \
-    g = (long long)sms * occ;                                                                               \
-    const long long need = (A.n + 7) / 8; /* 8 warps per CTA, one row each */                              \
-    if (g > need) g = need;                                                                                 \
-    if (g < 1) g = 1;                                                                                       \
-    kern<<<(unsigned)g, 256, 0, s>>>(A, Bv, ne, d_z, conj_z, P, V, A.n, m);                                 \
-  } while (0)
-#define SPF_VW(AC, BC, HB) \
-  do {                     \
-    if (vec2) SPF(AC, BC, HB, 2); else SPF(AC, BC, HB, 1); \
+  const CsrView Bv = B ? *B : A;
+  const int rows = kSpThreads / G;  // of a CTA
+  const int need = std::max(1, ceil_div(A.n, rows));
+  const size_t window = std::min<size_t>(A.n, (size_t)bw + (size_t)4 * sms * rows) * m * sizeof(cxf);
+  const int ng = (int)std::min<size_t>(ne, std::max<size_t>(1, kGatherBytes / window));
+  const bool few = A.nnz <= 5 * (int64_t)A.n;
+#define SPF(AC, BC, HB, U)                                                                              \
+  do {                                                                                                  \
+    auto kern = k_multishift_spmm_f32<AC, BC, HB, PAIR, G, U>;                                          \
+    int occ = 1;                                                                                        \
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSpThreads, 0);                           \
+    kern<<<std::min(occ * sms, need), kSpThreads, 0, s>>>(A, Bv, ne, d_z, conj_z, P, V, A.n, m, ng);    \
   } while (0)
   if (!B) {
-    if (A.cplx) SPF_VW(true, false, false); else SPF_VW(false, false, false);
-  } else if (bc) {
-    if (A.cplx) SPF_VW(true, true, true); else SPF_VW(false, true, true);
+    if (A.cplx) {
+      if (few) SPF(true, false, false, 5); else SPF(true, false, false, 9);
+    } else {
+      if (few) SPF(false, false, false, 5); else SPF(false, false, false, 9);
+    }
+  } else if (B->cplx) {
+    if (A.cplx) SPF(true, true, true, 5); else SPF(false, true, true, 5);
   } else {
-    if (A.cplx) SPF_VW(true, false, true); else SPF_VW(false, false, true);
+    if (A.cplx) SPF(true, false, true, 5); else SPF(false, false, true, 5);
   }
-#undef SPF_VW
 #undef SPF
-  return g;
+  note_launch();
+  return need;
 }
 
-int launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int ne, const cxd *d_z, int conj_z, const cxf *P,
-                               cxf *V, int m, int grid_per_sm, int max_row_nnz, cudaStream_t s) {
-  // register row length: the smallest that holds the longest row (longer
-  // rows and a non-identity B take the general loop of the same kernel)
-  long long g;
-  if (max_row_nnz <= 5) g = spmm_f32_dispatch<5>(A, B, ne, d_z, conj_z, P, V, m, grid_per_sm, s);
-  else if (max_row_nnz <= 7) g = spmm_f32_dispatch<7>(A, B, ne, d_z, conj_z, P, V, m, grid_per_sm, s);
-  else if (max_row_nnz <= 9) g = spmm_f32_dispatch<9>(A, B, ne, d_z, conj_z, P, V, m, grid_per_sm, s);
-  else g = spmm_f32_dispatch<16>(A, B, ne, d_z, conj_z, P, V, m, grid_per_sm, s);
-  note_launch();
-  return (int)g;
+int launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z, const cxf *P,
+                               cxf *V, int m, cudaStream_t s) {
+  // the fewest lanes a row that cover it in one pass
+  const int cols = ceil_div(m, 2);
+#define SPG(PAIR)                                                                            \
+  do {                                                                                       \
+    if (cols <= 4) return spmm_f32_launch<PAIR, 4>(A, B, bw, ne, d_z, conj_z, P, V, m, s);   \
+    if (cols <= 8) return spmm_f32_launch<PAIR, 8>(A, B, bw, ne, d_z, conj_z, P, V, m, s);   \
+    if (cols <= 16) return spmm_f32_launch<PAIR, 16>(A, B, bw, ne, d_z, conj_z, P, V, m, s); \
+    return spmm_f32_launch<PAIR, 32>(A, B, bw, ne, d_z, conj_z, P, V, m, s);                 \
+  } while (0)
+  if (m % 2 == 0) SPG(true);
+  SPG(false);
+#undef SPG
 }
