@@ -22,62 +22,94 @@ constexpr int kFgMaxK = 64;
 constexpr int kFgThreads = 256;
 }  // namespace
 
-// partial[chunk][l][s] = sum over the chunk's rows of conj(V_l) * w  (l < nv)
-__global__ void __launch_bounds__(kFgThreads) k_fg_dots(const cxf *const *V, int nv, const cxf *w, int ne, int n,
-                                                        int m, int rows_per_cta, const int *active, cxd *partial) {
-  const int S = ne * m;
+// One pass over w by row blocks held in registers:
+//   UPDATE  w -= sum_l h[l][s] V_l (the coefficients of the pass before),
+//   then partial[chunk][l][s] = sum over the chunk's rows of conj(V_l) w, or
+//   NORM    partial[chunk][s] = sum of |w|^2.
+// V_l = V + l vs.  Bound by reading V twice out of L2 (the second time mostly
+// out of L1).  A thread a system, kRB rows at a time: their loads are issued
+// together, and their sums enter the FP64 partials as one value, in two FP32
+// chains of four (as separate kernels, with as many chunks of rows as fit 8 CTAs
+// an SM and each V_l in a loop over single rows, an orthogonalisation with its
+// partial sums took 85 us a step at n = 3000, 192 systems, 44 us now).
+constexpr int kRB = 8;
+template <bool UPDATE, bool NORM>
+__global__ void __launch_bounds__(kFgThreads) k_fg_pass(const cxf *__restrict__ V, size_t vs, int nv,
+                                                        const cxd *__restrict__ h, cxf *w, int S, int n, int m,
+                                                        int rows_per_cta, const int *__restrict__ active,
+                                                        cxd *__restrict__ partial) {
+  const int s = blockIdx.y * kFgThreads + threadIdx.x;
+  if (s >= S || !active[s]) return;
   const int r0 = blockIdx.x * rows_per_cta, r1 = min(n, r0 + rows_per_cta);
-  for (int s = threadIdx.x; s < S; s += blockDim.x) {
-    if (!active[s]) continue;
-    const int j = s / m, c = s - j * m;
-    const size_t base = (size_t)j * n * m + c;
-    for (int l = 0; l < nv; ++l) {
-      const cxf *Vl = V[l];
-      cxf acc = mk(0.f, 0.f);
-      for (int i = r0; i < r1; ++i) cfma_cj(acc, Vl[base + (size_t)i * m], w[base + (size_t)i * m]);
-      partial[((size_t)blockIdx.x * nv + l) * S + s] = ccast<double>(acc);
-    }
-  }
-}
-// out[l][s] = sum over the chunks of partial (fixed order): one CTA per 2
-// outputs, 128 threads each.  A thread per output took 167 us at 1000 chunks
-// (three quarters of an FGMRES solve).
-constexpr int kFdC = 2, kFdR = 128;
-__global__ void __launch_bounds__(kFdC *kFdR) k_fg_dots_reduce(const cxd *__restrict__ partial, int nchunks, int count,
-                                                               cxd *out) {
-  __shared__ cxd sm[kFdC * kFdR];
-  const int e = blockIdx.x * kFdC + threadIdx.x % kFdC;
-  const cxd s = column_sum<kFdC, kFdR>(partial, nchunks, count, e, e < count, sm);
-  if (e < count && threadIdx.x < kFdC) out[e] = s;
-}
-static void fg_dots_reduce(const cxd *partial, int nchunks, int count, cxd *out, cudaStream_t s) {
-  k_fg_dots_reduce<<<ceil_div(count, kFdC), kFdC * kFdR, 0, s>>>(partial, nchunks, count, out);
-  note_launch();
-}
-// w -= sum_l h[l][s] V_l ; H[s][l][col] += h[l][s] (the Gram-Schmidt coefficients)
-__global__ void k_fg_orth_update(const cxf *const *V, int nv, const cxd *h, cxf *w, int ne, int n, int m,
-                                 const int *active, cxd *H, int kmax, int col) {
-  const int S = ne * m;
-  const size_t count = (size_t)ne * n * m;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t j = e / ((size_t)n * m), rem = e - j * n * m;
-    const int c = (int)(rem % m);
-    const int s = (int)j * m + c;
-    if (!active[s]) continue;
-    cxf acc = w[e];
-    for (int l = 0; l < nv; ++l) cfms(acc, ccast<float>(h[(size_t)l * S + s]), V[l][e]);
-    w[e] = acc;
-  }
-  if (blockIdx.x == 0)
-    for (int q = threadIdx.x; q < nv * S; q += blockDim.x) {
-      const int l = q / S, s = q - l * S;
-      if (active[s]) {
-        cxd &hv = H[((size_t)s * (kmax + 1) + l) * kmax + col];
-        hv = hv + h[q];
+  const int j = s / m, c = s - j * m;
+  for (int i = r0; i < r1; i += kRB) {
+    const size_t base = ((size_t)j * n + i) * m + c;
+    const int cnt = min(kRB, r1 - i);
+    cxf x[kRB];
+#pragma unroll
+    for (int r = 0; r < kRB; ++r) x[r] = r < cnt ? w[base + (size_t)r * m] : mk(0.f, 0.f);
+    if (UPDATE) {
+      for (int l = 0; l < nv; ++l) {
+        const cxf hl = ccast<float>(h[(size_t)l * S + s]);
+        const cxf *Vl = V + l * vs + base;
+        cxf v[kRB];
+#pragma unroll
+        for (int r = 0; r < kRB; ++r) v[r] = r < cnt ? Vl[(size_t)r * m] : mk(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < kRB; ++r) cfms(x[r], hl, v[r]);
       }
+#pragma unroll
+      for (int r = 0; r < kRB; ++r)
+        if (r < cnt) w[base + (size_t)r * m] = x[r];
     }
+    for (int l = 0; l < (NORM ? 1 : nv); ++l) {
+      cxf a0 = mk(0.f, 0.f), a1 = a0;
+      if (NORM) {
+#pragma unroll
+        for (int r = 0; r < kRB; r += 2) {
+          cfma_cj(a0, x[r], x[r]);
+          cfma_cj(a1, x[r + 1], x[r + 1]);
+        }
+      } else {
+        const cxf *Vl = V + l * vs + base;
+        cxf v[kRB];
+#pragma unroll
+        for (int r = 0; r < kRB; ++r) v[r] = r < cnt ? Vl[(size_t)r * m] : mk(0.f, 0.f);
+#pragma unroll
+        for (int r = 0; r < kRB; r += 2) {
+          cfma_cj(a0, v[r], x[r]);
+          cfma_cj(a1, v[r + 1], x[r + 1]);
+        }
+      }
+      cxd *o = partial + ((size_t)blockIdx.x * (NORM ? 1 : nv) + l) * S + s;
+      const cxd sum = ccast<double>(a0 + a1);
+      *o = i == r0 ? sum : *o + sum;
+    }
+  }
 }
-// per system: h_{col+1,col} = ||w|| (from the reduced |w|^2), v_{col+1} = w / h;
+// out[l][s] = sum over the chunks of partial (fixed order): one CTA per 8
+// outputs, 32 threads each (more threads an output spend the FP64 pipe on the tree).  A thread per output took 167 us at 1000 chunks
+// (three quarters of an FGMRES solve).  H (may be NULL): the Gram-Schmidt
+// coefficients, H[s][l][col] += out[l][s].
+constexpr int kFrC = 8, kFrR = 32;
+__global__ void __launch_bounds__(kFrC *kFrR) k_fg_dots_reduce(const cxd *__restrict__ partial, int nchunks, int count,
+                                                               cxd *out, int S, const int *active, cxd *H, int kmax,
+                                                               int col) {
+  __shared__ cxd sm[kFrC * kFrR];
+  const int e = blockIdx.x * kFrC + threadIdx.x % kFrC;
+  const int l = e / S, s = e - l * S;
+  const bool ok = e < count && active[s];
+  const cxd v = column_sum<kFrC, kFrR>(partial, nchunks, count, e, ok, sm);
+  if (ok && threadIdx.x < kFrC) {
+    out[e] = v;
+    if (H) {
+      cxd &hv = H[((size_t)s * (kmax + 1) + l) * kmax + col];
+      hv = hv + v;
+    }
+  }
+}
+constexpr int kFdC = 4, kFdR = 64;
+// per system: h_{col+1,col} = ||w|| (sum of the partials of |w|^2), v_{col+1} = w / h;
 // Givens rotations on column col, residual estimate, convergence
 struct FgScal {
   cxd *H;        // S x (kmax+1) x kmax
@@ -88,15 +120,20 @@ struct FgScal {
   int *active;   // still iterating
   int *nact;     // count of active systems after this step
 };
-__global__ void k_fg_arnoldi_tail(FgScal sc, const cxd *wn2, int S, int kmax, int col, double tol, cxd *invh) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  invh[s] = mk(0.0, 0.0);
-  if (!sc.active[s]) return;
-  const double hn = sqrt(fmax(wn2[s].re, 0.0));
+__global__ void __launch_bounds__(kFdC *kFdR)
+    k_fg_arnoldi_tail(FgScal sc, const cxd *__restrict__ partial, int nchunks, int S, int kmax, int col, double tol,
+                      cxf *invh) {
+  __shared__ cxd sm[kFdC * kFdR];
+  const int s = blockIdx.x * kFdC + threadIdx.x % kFdC;
+  const bool ok = s < S && sc.active[s];
+  const cxd wn2 = column_sum<kFdC, kFdR>(partial, nchunks, S, s, ok, sm);
+  if (threadIdx.x >= kFdC || s >= S) return;
+  invh[s] = mk(0.f, 0.f);
+  if (!ok) return;
+  const double hn = sqrt(fmax(wn2.re, 0.0));
   cxd *Hs = sc.H + (size_t)s * (kmax + 1) * kmax;
   Hs[(size_t)(col + 1) * kmax + col] = mk(hn, 0.0);
-  invh[s] = hn > 0 ? mk(1.0 / hn, 0.0) : mk(0.0, 0.0);
+  invh[s] = hn > 0 ? mk((float)(1.0 / hn), 0.f) : mk(0.f, 0.f);
   // apply the previous rotations to column col
   for (int l = 0; l < col; ++l) {
     const cxd c = sc.cs[(size_t)s * kmax + l], sn = sc.sn[(size_t)s * kmax + l];
@@ -133,56 +170,52 @@ __global__ void k_fg_arnoldi_tail(FgScal sc, const cxd *wn2, int S, int kmax, in
   if (sc.active[s]) atomicAdd(sc.nact, 1);
 }
 // v = w * invh (per system), only systems that got a new column
-__global__ void k_fg_scale(const cxf *w, const cxd *invh, cxf *v, int ne, int n, int m) {
+__global__ void k_fg_scale(const cxf *w, const cxf *invh, cxf *v, int ne, int n, int m) {
   const size_t count = (size_t)ne * n * m;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
     const size_t j = e / ((size_t)n * m), rem = e - j * n * m;
     const int s = (int)j * m + (int)(rem % m);
-    v[e] = ccast<float>(invh[s]) * w[e];
+    v[e] = invh[s] * w[e];
   }
 }
-// start of a cycle: beta = |r| per system, v0 = r / beta, g = (beta, 0, ...)
-__global__ void k_fg_start(FgScal sc, const cxd *rn2, int S, int kmax, double tol_abs_scale, const double *bnorm,
-                           double tol, cxd *invh) {
+// start of a cycle: beta = |r| per system, v0 = r / beta, g = (beta, 0, ...); H and
+// g were zeroed
+__global__ void k_fg_start(FgScal sc, const cxd *rn2, int S, int kmax, const double *bnorm, double tol, cxf *invh) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
   const double b = sqrt(fmax(rn2[s].re, 0.0));
   sc.beta[s] = bnorm ? bnorm[s] : b;
-  for (int q = 0; q < (kmax + 1) * kmax; ++q) sc.H[(size_t)s * (kmax + 1) * kmax + q] = mk(0.0, 0.0);
-  for (int q = 0; q <= kmax; ++q) sc.g[(size_t)s * (kmax + 1) + q] = mk(0.0, 0.0);
   sc.g[(size_t)s * (kmax + 1)] = mk(b, 0.0);
   sc.resid[s] = b;
   const bool go = b > tol * sc.beta[s] && b == b && b > 0;
   sc.active[s] = go ? 1 : 0;
-  invh[s] = go ? mk(1.0 / b, 0.0) : mk(0.0, 0.0);
+  invh[s] = go ? mk((float)(1.0 / b), 0.f) : mk(0.f, 0.f);
   if (go) atomicAdd(sc.nact, 1);
-  (void)tol_abs_scale;
 }
-// y = H^{-1} g (upper triangular, k columns) per system; y into ycoef[s][l]
-__global__ void k_fg_solve_small(FgScal sc, int S, int kmax, int k, const int *used, cxd *ycoef) {
+// y = H^{-1} g (upper triangular, k columns) per system; in FP32 into yf[l][s]
+__global__ void k_fg_solve_small(FgScal sc, int S, int kmax, int k, cxd *ycoef, cxf *yf) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
-  const int kk = used[s];
   const cxd *Hs = sc.H + (size_t)s * (kmax + 1) * kmax;
   const cxd *gs = sc.g + (size_t)s * (kmax + 1);
   cxd *y = ycoef + (size_t)s * kmax;
-  for (int l = 0; l < kmax; ++l) y[l] = mk(0.0, 0.0);
-  for (int l = kk - 1; l >= 0; --l) {
+  for (int l = k - 1; l >= 0; --l) {
     cxd acc = gs[l];
-    for (int q = l + 1; q < kk; ++q) cfms(acc, Hs[(size_t)l * kmax + q], y[q]);
+    for (int q = l + 1; q < k; ++q) cfms(acc, Hs[(size_t)l * kmax + q], y[q]);
     const cxd d = Hs[(size_t)l * kmax + l];
     y[l] = (abs2(d) > 0) ? cdiv(acc, d) : mk(0.0, 0.0);
+    yf[(size_t)l * S + s] = ccast<float>(y[l]);
   }
-  (void)k;
 }
-// d += sum_l y_l Z_l
-__global__ void k_fg_update_x(const cxf *const *Z, int k, const cxd *ycoef, int kmax, cxf *d, int ne, int n, int m) {
-  const size_t count = (size_t)ne * n * m;
+// d += sum_l y_l Z_l, Z_l = Z + l vs
+__global__ void k_fg_update_x(const cxf *__restrict__ Z, size_t vs, int k, const cxf *__restrict__ yf, int S, cxf *d,
+                              int n, int m, size_t count) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
     const size_t j = e / ((size_t)n * m), rem = e - j * n * m;
     const int s = (int)j * m + (int)(rem % m);
     cxf acc = d[e];
-    for (int l = 0; l < k; ++l) cfma(acc, ccast<float>(ycoef[(size_t)s * kmax + l]), Z[l][e]);
+#pragma unroll 4
+    for (int l = 0; l < k; ++l) cfma(acc, yf[(size_t)l * S + s], Z[l * vs + e]);
     d[e] = acc;
   }
 }
@@ -220,24 +253,23 @@ __global__ void __launch_bounds__(256) k_fg_jacobi(const cxf *__restrict__ v, co
 // ---------------------------------------------------------------------------
 // host driver
 // ---------------------------------------------------------------------------
+constexpr int kFgChunks = 1216;
+static size_t fg_block_bytes(int n, int m0, int ne) { return ((size_t)ne * n * m0 * sizeof(cxf) + 255) & ~(size_t)255; }
+
 size_t fgmres_work_bytes(int n, int m0, int ne, int kmax) {
-  const size_t blk = (size_t)ne * n * m0 * sizeof(cxf);
   const size_t S = (size_t)ne * m0;
-  const int chunks = 1216;
-  return (2 * (size_t)kmax + 4) * blk + (size_t)chunks * (kmax + 1) * S * sizeof(cxd) +
-         S * ((size_t)(kmax + 1) * kmax + 3 * kmax + 2 * (kmax + 1) + 8) * sizeof(cxd) + (64 << 10) +
-         2 * (size_t)(2 * kmax + 4) * sizeof(void *);
+  return (2 * (size_t)kmax + 4) * fg_block_bytes(n, m0, ne) + (size_t)kFgChunks * (kmax + 1) * S * sizeof(cxd) +
+         S * ((size_t)(kmax + 1) * kmax + 4 * kmax + 2 * (kmax + 1) + 8) * sizeof(cxd) + (64 << 10);
 }
 
 namespace {
 struct FgWork {
-  std::vector<cxf *> V, Z;
+  cxf *V, *Z;    // kmax + 1 and kmax blocks
+  size_t vs;     // entries from one block to the next
   cxf *w, *o, *r;
-  cxd *partial, *dots, *invh, *ycoef;
+  cxd *partial, *dots, *ycoef;
+  cxf *invh, *yf;
   FgScal sc;
-  int *used;
-  const cxf **dV, **dZ;
-  int chunks;
 };
 
 FgWork fg_carve(void *work, int n, int m0, int ne, int kmax) {
@@ -248,20 +280,19 @@ FgWork fg_carve(void *work, int n, int m0, int ne, int kmax) {
     p += (bytes + 255) & ~(size_t)255;
     return q;
   };
-  const size_t blk = (size_t)ne * n * m0 * sizeof(cxf);
+  const size_t blk = fg_block_bytes(n, m0, ne);
   const size_t S = (size_t)ne * m0;
-  f.chunks = 1216;
-  f.V.resize(kmax + 1);
-  f.Z.resize(kmax);
-  for (int l = 0; l <= kmax; ++l) f.V[l] = (cxf *)take(blk);
-  for (int l = 0; l < kmax; ++l) f.Z[l] = (cxf *)take(blk);
+  f.vs = blk / sizeof(cxf);
+  f.V = (cxf *)take((kmax + 1) * blk);
+  f.Z = (cxf *)take(kmax * blk);
   f.w = (cxf *)take(blk);
   f.o = (cxf *)take(blk);
   f.r = (cxf *)take(blk);
-  f.partial = (cxd *)take((size_t)f.chunks * (kmax + 1) * S * sizeof(cxd));
+  f.partial = (cxd *)take((size_t)kFgChunks * (kmax + 1) * S * sizeof(cxd));
   f.dots = (cxd *)take((kmax + 1) * S * sizeof(cxd));
-  f.invh = (cxd *)take(S * sizeof(cxd));
+  f.invh = (cxf *)take(S * sizeof(cxf));
   f.ycoef = (cxd *)take(S * kmax * sizeof(cxd));
+  f.yf = (cxf *)take(S * kmax * sizeof(cxf));
   f.sc.H = (cxd *)take(S * (kmax + 1) * kmax * sizeof(cxd));
   f.sc.cs = (cxd *)take(S * kmax * sizeof(cxd));
   f.sc.sn = (cxd *)take(S * kmax * sizeof(cxd));
@@ -270,20 +301,30 @@ FgWork fg_carve(void *work, int n, int m0, int ne, int kmax) {
   f.sc.resid = (double *)take(S * sizeof(double));
   f.sc.active = (int *)take(S * sizeof(int));
   f.sc.nact = (int *)take(64);
-  f.used = (int *)take(S * sizeof(int));
-  f.dV = (const cxf **)take((kmax + 1) * sizeof(void *));
-  f.dZ = (const cxf **)take(kmax * sizeof(void *));
   return f;
 }
 
-void fg_dots(FgWork &f, int nv, const cxf *w, int ne, int n, int m, cudaStream_t s) {
-  const int S = ne * m;
-  int chunks = std::min(f.chunks, n);
-  const int rpc = ceil_div(n, chunks);
-  chunks = ceil_div(n, rpc);
-  k_fg_dots<<<chunks, kFgThreads, 0, s>>>(f.dV, nv, w, ne, n, m, rpc, f.sc.active, f.partial);
+// Rows of a CTA: one block of kRB where that is no more than kFgChunks chunks.
+int fg_rows(int n) { return ceil_div(ceil_div(n, kFgChunks), kRB) * kRB; }
+
+template <bool UPDATE, bool NORM>
+int fg_pass(FgWork &f, int nv, cxf *w, int S, int n, int m, cudaStream_t s) {
+  const int rpc = fg_rows(n), chunks = ceil_div(n, rpc);
+  k_fg_pass<UPDATE, NORM><<<dim3(chunks, ceil_div(S, kFgThreads)), kFgThreads, 0, s>>>(
+      f.V, f.vs, nv, f.dots, w, S, n, m, rpc, f.sc.active, f.partial);
   note_launch();
-  fg_dots_reduce(f.partial, chunks, nv * S, f.dots, s);
+  return chunks;
+}
+void fg_reduce(FgWork &f, int chunks, int nv, int S, bool coef, int kmax, int col, cudaStream_t s) {
+  k_fg_dots_reduce<<<ceil_div(nv * S, kFrC), kFrC * kFrR, 0, s>>>(f.partial, chunks, nv * S, f.dots, S, f.sc.active,
+                                                                  coef ? f.sc.H : nullptr, kmax, col);
+  note_launch();
+}
+// |x|^2 of every system into dots (all systems active)
+void fg_norms(FgWork &f, const cxf *x, int S, int n, int m, cudaStream_t s) {
+  cudaMemsetAsync(f.sc.active, 1, S * sizeof(int), s);  // any non-zero value
+  const int chunks = fg_pass<false, true>(f, 1, const_cast<cxf *>(x), S, n, m, s);
+  fg_reduce(f, chunks, 1, S, false, 0, 0, s);
 }
 }  // namespace
 
@@ -294,23 +335,10 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
   const int S = ne * m;
   const size_t count = (size_t)ne * n * m;
   const unsigned gb = grid_for(count);
-  // device arrays of block pointers
-  std::vector<const cxf *> hv(f.V.begin(), f.V.end()), hz(f.Z.begin(), f.Z.end());
-  cudaMemcpyAsync(f.dV, hv.data(), hv.size() * sizeof(void *), cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(f.dZ, hz.data(), hz.size() * sizeof(void *), cudaMemcpyHostToDevice, s);
-  // |b| per system (the convergence reference), via the dot kernel on b, b
   cudaMemsetAsync(d, 0, count * sizeof(cxf), s);
-  // all systems active for the norm of b
-  std::vector<int> ones(S, 1);
-  cudaMemcpyAsync(f.sc.active, ones.data(), S * sizeof(int), cudaMemcpyHostToDevice, s);
   cudaMemcpyAsync(f.r, b, count * sizeof(cxf), cudaMemcpyDeviceToDevice, s);
-  {
-    const cxf *vb[1] = {b};
-    cudaMemcpyAsync(f.dV, vb, sizeof(void *), cudaMemcpyHostToDevice, s);
-    fg_dots(f, 1, b, ne, n, m, s);
-  }
-  // keep |b|^2 in partial-free storage: beta of the first start is |b|
-  cudaMemcpyAsync(f.dV, hv.data(), hv.size() * sizeof(void *), cudaMemcpyHostToDevice, s);
+  // |b| per system, the convergence reference: beta of the first start
+  fg_norms(f, b, S, n, m, s);
   int its = 0;
   int h_nact = 0;
   bool first = true;
@@ -320,53 +348,37 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
       op.apply(op.ctx, d, f.o, s);
       k_fg_sub<<<gb, 256, 0, s>>>(b, f.o, f.r, count);
       note_launch();
-      cudaMemcpyAsync(f.sc.active, ones.data(), S * sizeof(int), cudaMemcpyHostToDevice, s);
-      const cxf *vr[1] = {f.r};
-      cudaMemcpyAsync(f.dV, vr, sizeof(void *), cudaMemcpyHostToDevice, s);
-      fg_dots(f, 1, f.r, ne, n, m, s);
-      cudaMemcpyAsync(f.dV, hv.data(), hv.size() * sizeof(void *), cudaMemcpyHostToDevice, s);
+      fg_norms(f, f.r, S, n, m, s);
     }
     cudaMemsetAsync(f.sc.nact, 0, sizeof(int), s);
+    cudaMemsetAsync(f.sc.H, 0, (size_t)S * (kmax + 1) * kmax * sizeof(cxd), s);
+    cudaMemsetAsync(f.sc.g, 0, (size_t)S * (kmax + 1) * sizeof(cxd), s);
     // beta of the first cycle is |b| itself (kept in sc.beta across cycles)
-    k_fg_start<<<ceil_div(S, 128), 128, 0, s>>>(f.sc, f.dots, S, kmax, 0.0, first ? nullptr : f.sc.beta, tol,
-                                                f.invh);
+    k_fg_start<<<ceil_div(S, 128), 128, 0, s>>>(f.sc, f.dots, S, kmax, first ? nullptr : f.sc.beta, tol, f.invh);
     note_launch();
     first = false;
-    k_fg_scale<<<gb, 256, 0, s>>>(f.r, f.invh, f.V[0], ne, n, m);
+    k_fg_scale<<<gb, 256, 0, s>>>(f.r, f.invh, f.V, ne, n, m);
     note_launch();
     cudaMemcpyAsync(&h_nact, f.sc.nact, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaStreamSynchronize(s);
     if (h_nact == 0) break;
     int col = 0;
     for (col = 0; col < kmax && its < maxit; ++col, ++its) {
-      op.precond(op.ctx, f.V[col], f.Z[col], s);
-      op.apply(op.ctx, f.Z[col], f.w, s);
-      for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
-        fg_dots(f, col + 1, f.w, ne, n, m, s);
-        k_fg_orth_update<<<gb, 256, 0, s>>>(f.dV, col + 1, f.dots, f.w, ne, n, m, f.sc.active, f.sc.H, kmax, col);
-        note_launch();
-      }
-      {
-        const cxf *vw[1] = {f.w};
-        cudaMemcpyAsync(f.dV + kmax, vw, sizeof(void *), cudaMemcpyHostToDevice, s);
-      }
-      // |w|^2 through the dot kernel with V_kmax := w
-      {
-        const cxf **dv = f.dV + kmax;
-        const int chunks = ceil_div(n, ceil_div(n, std::min(f.chunks, n)));
-        const int rpc = ceil_div(n, chunks);
-        k_fg_dots<<<chunks, kFgThreads, 0, s>>>(dv, 1, f.w, ne, n, m, rpc, f.sc.active, f.partial);
-        note_launch();
-        fg_dots_reduce(f.partial, chunks, S, f.dots, s);
-      }
-      cudaMemcpyAsync(f.dV + kmax, &hv[kmax], sizeof(void *), cudaMemcpyHostToDevice, s);
+      op.precond(op.ctx, f.V + col * f.vs, f.Z + col * f.vs, s);
+      op.apply(op.ctx, f.Z + col * f.vs, f.w, s);
+      // classical Gram-Schmidt, twice
+      int chunks = fg_pass<false, false>(f, col + 1, f.w, S, n, m, s);
+      fg_reduce(f, chunks, col + 1, S, true, kmax, col, s);
+      fg_pass<true, false>(f, col + 1, f.w, S, n, m, s);
+      fg_reduce(f, chunks, col + 1, S, true, kmax, col, s);
+      fg_pass<true, true>(f, col + 1, f.w, S, n, m, s);
       cudaMemsetAsync(f.sc.nact, 0, sizeof(int), s);
-      k_fg_arnoldi_tail<<<ceil_div(S, 128), 128, 0, s>>>(f.sc, f.dots, S, kmax, col, tol, f.invh);
+      k_fg_arnoldi_tail<<<ceil_div(S, kFdC), kFdC * kFdR, 0, s>>>(f.sc, f.partial, chunks, S, kmax, col, tol, f.invh);
       note_launch();
-      k_fg_scale<<<gb, 256, 0, s>>>(f.w, f.invh, f.V[col + 1], ne, n, m);
+      k_fg_scale<<<gb, 256, 0, s>>>(f.w, f.invh, f.V + (col + 1) * f.vs, ne, n, m);
       note_launch();
-      // used columns per system: every system uses col + 1 columns this cycle
-      // (frozen systems have zero rows in H and g beyond their last column)
+      // every system uses col + 1 columns this cycle (frozen systems have zero
+      // rows in H and g beyond their last column)
       cudaMemcpyAsync(&h_nact, f.sc.nact, sizeof(int), cudaMemcpyDeviceToHost, s);
       cudaStreamSynchronize(s);
       if (h_nact == 0) {
@@ -376,11 +388,9 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
       }
     }
     // d += Z y with y = H^{-1} g over the columns built in this cycle
-    std::vector<int> used(S, col);
-    cudaMemcpyAsync(f.used, used.data(), S * sizeof(int), cudaMemcpyHostToDevice, s);
-    k_fg_solve_small<<<ceil_div(S, 128), 128, 0, s>>>(f.sc, S, kmax, col, f.used, f.ycoef);
+    k_fg_solve_small<<<ceil_div(S, 128), 128, 0, s>>>(f.sc, S, kmax, col, f.ycoef, f.yf);
     note_launch();
-    k_fg_update_x<<<gb, 256, 0, s>>>(f.dZ, col, f.ycoef, kmax, d, ne, n, m);
+    k_fg_update_x<<<gb, 256, 0, s>>>(f.Z, f.vs, col, f.yf, S, d, n, m, count);
     note_launch();
     if (h_nact == 0) break;
   }
@@ -388,12 +398,7 @@ int fgmres_solve(const FgmresOp &op, const cxf *b, cxf *d, int n, int m, int ne,
   op.apply(op.ctx, d, f.o, s);
   k_fg_sub<<<gb, 256, 0, s>>>(b, f.o, f.r, count);
   note_launch();
-  cudaMemcpyAsync(f.sc.active, ones.data(), S * sizeof(int), cudaMemcpyHostToDevice, s);
-  {
-    const cxf *vr[1] = {f.r};
-    cudaMemcpyAsync(f.dV, vr, sizeof(void *), cudaMemcpyHostToDevice, s);
-    fg_dots(f, 1, f.r, ne, n, m, s);
-  }
+  fg_norms(f, f.r, S, n, m, s);
   std::vector<cxd> rr(S);
   std::vector<double> bb(S);
   cudaMemcpyAsync(rr.data(), f.dots, S * sizeof(cxd), cudaMemcpyDeviceToHost, s);
