@@ -268,8 +268,12 @@ __global__ void __launch_bounds__(512) k_band_panel_reg(int n, int kl, int ku, i
   }
 }
 
-// U12 = L11^{-1} A12 for the panel at column k, one column per thread (no
-// barrier): rows [k, k+nb), columns [k+nb, k+nb+ku).  grid (ceil(ku/128), ne).
+// U12 = L11^{-1} A12 for the panel at column k: rows [k, k+nb), columns
+// [k+nb, k+nb+ku).  NB lanes a column, a row each; the solved entries are
+// passed on by shuffles.  grid (ceil(ku / (128 / NB)), ne).  An FP64 warp
+// instruction takes its pipe 64 cycles whatever its lanes, so a column a
+// thread, with all of the column's products in one warp, took 18 us a panel
+// at ku = 40, U12US now.
 template <typename T, int NB>
 __global__ void __launch_bounds__(128) k_band_u12(int n, int kl, int ku, int k, cx<T> *band, size_t ns) {
   __shared__ cx<T> L11[NB][NB + 1];
@@ -283,29 +287,23 @@ __global__ void __launch_bounds__(128) k_band_u12(int n, int kl, int ku, int k, 
     L11[r][p] = (r < nb && p < r && -d <= kl) ? Bd[(size_t)(k + r) * W + (d + kl)] : mk<T>(0, 0);
   }
   __syncthreads();
-  const int c2 = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c2 >= ucol) return;
-  cx<T> col[NB];
+  const int r = threadIdx.x % NB, c2 = blockIdx.x * (128 / NB) + threadIdx.x / NB;
+  const int d = nb + c2 - r;
+  const bool in = c2 < ucol && r < nb && d <= ku;
+  cx<T> x = in ? Bd[(size_t)(k + r) * W + (d + kl)] : mk<T>(0, 0);
 #pragma unroll
-  for (int r = 0; r < NB; ++r) {
-    const int d = nb + c2 - r;
-    col[r] = (r < nb && d <= ku) ? Bd[(size_t)(k + r) * W + (d + kl)] : mk<T>(0, 0);
+  for (int p = 0; p < NB - 1; ++p) {
+    const cx<T> v = mk<T>(__shfl_sync(0xffffffffu, x.re, p, NB), __shfl_sync(0xffffffffu, x.im, p, NB));
+    if (r > p) cfms(x, L11[r][p], v);
   }
-#pragma unroll
-  for (int r = 1; r < NB; ++r)
-#pragma unroll
-    for (int p = 0; p < r; ++p) cfms(col[r], L11[r][p], col[p]);
-#pragma unroll
-  for (int r = 0; r < NB; ++r) {
-    const int d = nb + c2 - r;
-    if (r < nb && d <= ku) Bd[(size_t)(k + r) * W + (d + kl)] = col[r];
-  }
+  if (in) Bd[(size_t)(k + r) * W + (d + kl)] = x;
 }
 
-// Trailing update A22 -= L21 * U12 on rows [k+nb, k+nb+kl) x cols [k+nb, k+nb+ku).
-template <typename T, int NB>
+// Trailing update A22 -= L21 * U12 on rows [k+nb, k+nb+kl) x cols [k+nb, k+nb+ku),
+// in tiles of 16 E rows and columns, E x E entries a thread.
+template <typename T, int NB, int E>
 __global__ void __launch_bounds__(256) k_band_update(int n, int kl, int ku, int k, cx<T> *band, size_t ns) {
-  constexpr int TM = 64, TN = 64;
+  constexpr int TM = 16 * E, TN = 16 * E;
   __shared__ cx<T> Ls[TM][NB + 1];
   __shared__ cx<T> Us[NB][TN];
   const int W = kl + ku + 1;
@@ -331,34 +329,53 @@ __global__ void __launch_bounds__(256) k_band_update(int n, int kl, int ku, int 
   }
   __syncthreads();
   const int ty = tid >> 4, tx = tid & 15;
-  cx<T> acc[4][4];
+  cx<T> acc[E][E];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < E; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mk<T>(0, 0);
+    for (int j = 0; j < E; ++j) acc[i][j] = mk<T>(0, 0);
   for (int p = 0; p < nb; ++p) {
-    cx<T> a[4], b[4];
+    cx<T> a[E], b[E];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = Ls[ty + 16 * i][p];
+    for (int i = 0; i < E; ++i) a[i] = Ls[ty + 16 * i][p];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = Us[p][tx + 16 * j];
+    for (int j = 0; j < E; ++j) b[j] = Us[p][tx + 16 * j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < E; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], b[j]);
+      for (int j = 0; j < E; ++j) cfma(acc[i][j], a[i], b[j]);
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < E; ++i) {
     int r = r0 + ty + 16 * i;
     if (r >= r_end) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < E; ++j) {
       int c = c0 + tx + 16 * j;
       if (c >= c_end) continue;
       cx<T> &e = Bd[(size_t)r * W + (c - r + kl)];
       e = e - acc[i][j];
     }
   }
+}
+// The largest tile that still gives two CTAs an SM: 8 windows of 40 x 40 are 8
+// tiles of 64 x 64 (with 2.6 times the work, an SM each: 71 us a panel in FP64),
+// or 72 of 16 x 16 (UPDUS).
+template <typename T, int NB>
+static void launch_band_update(int n, int kl, int ku, int k, int rows, int cols, int ne, cx<T> *band, size_t ns,
+                               cudaStream_t s) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  auto ctas = [&](int t) { return (long long)ceil_div(cols, t) * ceil_div(rows, t) * ne; };
+  auto grid = [&](int t) { return dim3(ceil_div(cols, t), ceil_div(rows, t), ne); };
+  if (ctas(64) >= 2 * sms)
+    k_band_update<T, NB, 4><<<grid(64), 256, 0, s>>>(n, kl, ku, k, band, ns);
+  else if (ctas(32) >= 2 * sms)
+    k_band_update<T, NB, 2><<<grid(32), 256, 0, s>>>(n, kl, ku, k, band, ns);
+  else
+    k_band_update<T, NB, 1><<<grid(16), 256, 0, s>>>(n, kl, ku, k, band, ns);
+  note_launch();
 }
 
 // ---------------------------------------------------------------------------
@@ -670,7 +687,7 @@ cudaError_t band_factor(int n, int kl, int ku, int ne, cx<T> *band, int *d_err, 
       note_launch();
       const int ucol = min(n - k - min(NB, n - k), ku);
       if (ucol > 0) {
-        k_band_u12<T, NB><<<dim3(ceil_div(ucol, 128), ne), 128, 0, s>>>(n, kl, ku, k, band, ns);
+        k_band_u12<T, NB><<<dim3(ceil_div(ucol, 128 / NB), ne), 128, 0, s>>>(n, kl, ku, k, band, ns);
         note_launch();
       }
     } else {
@@ -680,11 +697,7 @@ cudaError_t band_factor(int n, int kl, int ku, int ne, cx<T> *band, int *d_err, 
     const int nb = min(NB, n - k);
     const int rows = min(n, k + nb + kl) - (k + nb);
     const int cols = min(n, k + nb + ku) - (k + nb);
-    if (rows > 0 && cols > 0) {
-      dim3 grid(ceil_div(cols, 64), ceil_div(rows, 64), ne);
-      k_band_update<T, NB><<<grid, 256, 0, s>>>(n, kl, ku, k, band, ns);
-      note_launch();
-    }
+    if (rows > 0 && cols > 0) launch_band_update<T, NB>(n, kl, ku, k, rows, cols, ne, band, ns, s);
   }
   return cudaGetLastError();
 }
