@@ -506,9 +506,9 @@ cudaError_t csr_transpose(const CsrView &A, int32_t *rowptr_t, int32_t *colind_t
 // third of L2.  Rows of up to U entries keep them in registers for all nodes.
 // 8 nodes of 50021 rows, 9 random entries each, 48 columns of P (154 MB):
 // 203 us with all nodes at once and a warp a row, 185 without the registers,
-// 149 us (the gathers are 1.5 GB, 10 TB/s out of L2); its transpose, with rows
-// of up to 25 entries, 352 -> 248 us; 200000 rows, 16 columns 654 -> 330; the
-// 300 x 300 grid, 16 columns 124 -> 51, 48 columns 144 -> 154.
+// 141 us (the gathers are 1.5 GB, 11 TB/s out of L2); its transpose, with rows
+// of up to 25 entries, 352 -> 248 us; 200000 rows, 16 columns 654 -> 330; on the
+// 300 x 300 grid, 16 columns 124 -> 50, 63 columns 281 -> 175.
 // ---------------------------------------------------------------------------
 // Two columns a lane: neighbours (PAIR, rows start on 16 bytes), or G apart
 // where m is odd.
@@ -608,7 +608,8 @@ __global__ void __launch_bounds__(kSpThreads, U == 5 ? 4 : PAIR ? 3 : 2)
       const bool row = i < n;
       const int64_t ka = row ? A.rowptr[i] : 0, kb = HASB && row ? B.rowptr[i] : 0;
       const int na = row ? (int)(A.rowptr[i + 1] - ka) : 0, nb = HASB && row ? (int)(B.rowptr[i + 1] - kb) : 0;
-      const int ma = __reduce_max_sync(0xffffffffu, na), mb = HASB ? __reduce_max_sync(0xffffffffu, nb) : 0;
+      const int ma = G == 32 ? na : __reduce_max_sync(0xffffffffu, na);
+      const int mb = !HASB || G == 32 ? nb : __reduce_max_sync(0xffffffffu, nb);
       RowPart<ACPLX, G> ra;  // -A
       RowPart<BCPLX, G> rb;
       ra.load(A, ka, na, 0, -1.f);
@@ -632,11 +633,9 @@ __global__ void __launch_bounds__(kSpThreads, U == 5 ? 4 : PAIR ? 3 : 2)
           for (int j = j0; j < j1; ++j) {
             const cxf *Pc = P + (size_t)j * xns + c;
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f), x[kShort];
-            const float4 own = load2<PAIR, G>(Pc + (size_t)i * m, second);
 #pragma unroll
-            for (int u = 0; u < kShort; ++u) {
-              x[u] = load2<PAIR, G>(Pc + (size_t)col[u] * m, second);
-            }
+            for (int u = 0; u < kShort; ++u) x[u] = load2<PAIR, G>(Pc + (size_t)col[u] * m, second);
+            const float4 own = load2<PAIR, G>(Pc + (size_t)i * m, second);
 #pragma unroll
             for (int u = 0; u < kShort; ++u) vfma<ACPLX>(acc, v[u], x[u]);
             vfma<true>(acc, zs[j], own);
@@ -672,7 +671,79 @@ __global__ void __launch_bounds__(kSpThreads, U == 5 ? 4 : PAIR ? 3 : 2)
 }
 
 
-constexpr size_t kGatherBytes = 40u << 20;
+// Rows of up to five entries, more than 32 columns (even), no B, all nodes at
+// once: a warp a row, whose entries every lane reads itself.  16 nodes, 64
+// columns of the 300 x 300 grid 291 us and 48 columns, 8 nodes 144 us, against
+// 320 and 162 with the lanes' entries above; longer rows take the loop.
+template <bool ACPLX>
+__global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView A, int ne, const cxd *__restrict__ z,
+                                                                         int conj_z, const cxf *__restrict__ P,
+                                                                         cxf *__restrict__ V, int n, int m) {
+  constexpr int K = 5;
+  __shared__ cxf zs[kMaxNe];
+  if (threadIdx.x < ne) {
+    const cxd zz = z[threadIdx.x];
+    zs[threadIdx.x] = mk((float)zz.re, conj_z ? -(float)zz.im : (float)zz.im);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int warp = (int)(((long long)blockIdx.x * kSpThreads + threadIdx.x) >> 5);
+  const int nwarps = (int)(((long long)gridDim.x * kSpThreads) >> 5);
+  const size_t xns = (size_t)n * m;
+  auto entry = [&](int64_t k) {  // of A
+    if constexpr (ACPLX) {
+      const cxd v = reinterpret_cast<const cxd *>(A.val)[k];
+      return mk((float)v.re, A.conj_vals ? -(float)v.im : (float)v.im);
+    }
+    return mk((float)A.val[k], 0.f);
+  };
+  auto sub = [](float4 &acc, cxf a, const float4 &x) {  // acc -= a x
+    acc.x = fmaf(-a.re, x.x, acc.x);
+    acc.x = fmaf(a.im, x.y, acc.x);
+    acc.y = fmaf(-a.re, x.y, acc.y);
+    acc.y = fmaf(-a.im, x.x, acc.y);
+    acc.z = fmaf(-a.re, x.z, acc.z);
+    acc.z = fmaf(a.im, x.w, acc.z);
+    acc.w = fmaf(-a.re, x.w, acc.w);
+    acc.w = fmaf(-a.im, x.z, acc.w);
+  };
+  for (int i = warp; i < n; i += nwarps) {
+    const int64_t ka = A.rowptr[i];
+    const int nk = (int)(A.rowptr[i + 1] - ka);
+    int col[K];
+    cxf av[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      col[k] = k < nk ? A.colind[ka + k] : i;
+      av[k] = k < nk ? entry(ka + k) : mk(0.f, 0.f);
+    }
+    const bool fast = nk <= K;
+    for (int c = lane * 2; c < m; c += 64) {
+#pragma unroll 2
+      for (int j = 0; j < ne; ++j) {
+        const cxf *Pj = P + (size_t)j * xns;
+        float4 acc;
+        acc.x = acc.y = 0.f;
+        acc.z = acc.w = 0.f;
+        if (fast) {
+          float4 xs[K];
+#pragma unroll
+          for (int k = 0; k < K; ++k) xs[k] = *reinterpret_cast<const float4 *>(Pj + (size_t)col[k] * m + c);
+          vfma<true>(acc, zs[j], *reinterpret_cast<const float4 *>(Pj + (size_t)i * m + c));
+#pragma unroll
+          for (int k = 0; k < K; ++k) sub(acc, av[k], xs[k]);
+        } else {
+          vfma<true>(acc, zs[j], *reinterpret_cast<const float4 *>(Pj + (size_t)i * m + c));
+          for (int k = 0; k < nk; ++k)
+            sub(acc, entry(ka + k), *reinterpret_cast<const float4 *>(Pj + (size_t)A.colind[ka + k] * m + c));
+        }
+        *reinterpret_cast<float4 *>(V + (size_t)j * xns + (size_t)i * m + c) = acc;
+      }
+    }
+  }
+}
+
+constexpr size_t kGatherBytes = 48u << 20;
 
 template <bool PAIR, int G>
 static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z, const cxf *P,
@@ -686,6 +757,21 @@ static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, c
   const size_t window = std::min<size_t>(A.n, (size_t)bw + (size_t)4 * sms * rows) * m * sizeof(cxf);
   const int ng = (int)std::min<size_t>(ne, std::max<size_t>(1, kGatherBytes / window));
   const bool few = A.nnz <= 5 * (int64_t)A.n;
+  if constexpr (PAIR && G == 32) {
+    if (few && !B && ng == ne) {
+      auto launch = [&](auto kern) {
+        int occ = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSpThreads, 0);
+        kern<<<std::min(occ * sms, need), kSpThreads, 0, s>>>(A, ne, d_z, conj_z, P, V, A.n, m);
+      };
+      if (A.cplx)
+        launch(k_multishift_spmm_f32_wide<true>);
+      else
+        launch(k_multishift_spmm_f32_wide<false>);
+      note_launch();
+      return need;
+    }
+  }
 #define SPF(AC, BC, HB, U)                                                                              \
   do {                                                                                                  \
     auto kern = k_multishift_spmm_f32<AC, BC, HB, PAIR, G, U>;                                          \

@@ -19,7 +19,7 @@ from gpu_helpers import host  # noqa: E402
     (1, 1, 2, 1, False, False), (40, 2, 3, 2, True, False), (41, 7, 3, 30, False, False), (100, 8, 4, 4, False, True),
     (101, 10, 3, 4, True, True), (130, 16, 2, 6, False, False), (131, 17, 2, 12, True, False),
     (200, 33, 2, 70, False, True), (201, 34, 3, 40, True, False), (300, 66, 2, 5, False, False),
-    (56000, 96, 3, 3, False, False)])
+    (150, 40, 3, 3, True, False), (56000, 96, 3, 3, False, False), (56000, 96, 3, 7, False, False)])
 def test_operator(side, n, m, ne, per_row, cplx, withB):
     rng = np.random.default_rng(n + m)
 
