@@ -256,7 +256,7 @@ __global__ void k_block_entries(CsrView A, CsrView B, int hasB, int b, int K, in
 template <typename T>
 __global__ void __launch_bounds__(256) k_block_inv(int n, int kl, int ku, int b, const cx<T> *__restrict__ band,
                                                    size_t ns, const cx<T> *__restrict__ dinv, cx<T> *__restrict__ Tc,
-                                                   cx<T> *__restrict__ Tr) {
+                                                   cx<T> *__restrict__ Tr) {  // grid (blocks, column strips, slots)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int LDY = 33;
   cx<T> *Y = reinterpret_cast<cx<T> *>(smem_raw);  // b x LDY
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256) k_block_inv(int n, int kl, int ku, int b,
   cx<T> *P = F + (size_t)16 * (b + 2);             // 2 x 16 x 32 partial sums
   cx<T> *D = P + 2 * 16 * 32;                      // 16 x 17
   const int ldf = b + 2;
-  const int c0 = blockIdx.x * 32, blk = blockIdx.y, slot = blockIdx.z;
+  const int c0 = blockIdx.y * 32, blk = blockIdx.x, slot = blockIdx.z;
   const int W = kl + ku + 1, r0 = blk * b;
   const cx<T> *Bd = band + (size_t)slot * ns;
   const cx<T> *Dv = dinv + (size_t)slot * ceil_div(n, 16) * 1024;
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(256) k_block_inv(int n, int kl, int ku, int b,
       __syncthreads();
     }
   }
-  const size_t base = ((size_t)slot * gridDim.y + blk) * b * b;
+  const size_t base = ((size_t)slot * gridDim.x + blk) * b * b;
   for (int e = tid; e < b * 32; e += 256) {
     const int r = e >> 5, c = e & 31;
     if (c0 + c < b) put(Tr + base, b, r, c0 + c, Y[r * LDY + c]);
@@ -633,7 +633,8 @@ cudaError_t block_invert(int n, int kl, int ku, int klp, int kup, int nf, const 
   auto kern = k_block_inv<T>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_bytes<T>(b));
   if (e != cudaSuccess) return e;
-  kern<<<dim3(ceil_div(b, 32), ceil_div(n, b), nf), 256, inv_bytes<T>(b), s>>>(
+  // the blocks on x: more than 65535 of them (the limit of y) from n = 1048561 with blocks of 16
+  kern<<<dim3(ceil_div(n, b), ceil_div(b, 32), nf), 256, inv_bytes<T>(b), s>>>(
       n, klp, kup, b, band, (size_t)n * (klp + kup + 1), dinv, Tc, Tr);
   note_launch();
   return cudaGetLastError();

@@ -1,0 +1,37 @@
+"""Shifted solves at the ends of what the block form accepts (csrc/blocksolve.cu)."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+import scipy.sparse.linalg as spl
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+from paper_1506_04463_gb300 import feast_nh as F  # noqa: E402
+from paper_1506_04463_gb300 import workloads as wl  # noqa: E402
+from gpu_helpers import dev, host  # noqa: E402
+
+TOL = 1e-10
+
+
+@pytest.mark.parametrize("prec", [F.PREC_FP32_IR, F.PREC_FP64])
+def test_more_blocks_than_a_grid_has_rows(prec):
+    """Blocks of 16 rows, 65537 of them: more than the y and z extents of a grid take.  Entries below 0.2 off a
+    diagonal of 8, nodes at distance one from 4: ||M^{-1}|| <= 1 / (8 - 4 - 1 - 0.8) by rows and by columns, and the
+    two weights have modulus 1/2."""
+    n, m = 16 * 65536 + 1, 1
+    rng = np.random.default_rng(5)
+    A = (sp.diags([0.2 * rng.uniform(-1, 1, n - abs(o)) for o in (-2, -1, 1, 2)], (-2, -1, 1, 2)) + 8 * sp.eye(n)).tocsr()
+    con = wl.Contour(0, 4 + 0j, 1.0, ne=2)
+    Y = [rng.standard_normal((n, m)) + 1j * rng.standard_normal((n, m)) for _ in range(2)]
+    ctx = F.FeastNH(A, None, con, m, precision=prec, inner_tol=TOL)
+    out = [host(t) for t in ctx.filter(*(dev(y) for y in Y))]
+    ctx.close()
+    z, w = F.nodes(con)
+    lu = [spl.splu((zj * sp.eye(n) - A).tocsc()) for zj in z]
+    for side in range(2):
+        ref = sum((np.conj(wj) if side else wj) * f.solve(Y[side], trans="H" if side else "N") for f, wj in zip(lu, w))
+        err = np.linalg.norm(out[side] - ref, axis=0)
+        assert np.all(err <= (TOL + 1e-13) / 2.2 * np.linalg.norm(Y[side], axis=0)), (side, err.max())
