@@ -25,8 +25,15 @@
  *    feast_nh_rr and feast_nh_solve read a few numbers back from the device
  *    (inner residual and error word, subspace size, counts, convergence flag)
  *    once per call / per outer iteration / per refinement step.
- *  - The library allocates its workspace in feast_nh_init (and, for the
- *    banded factors, on the first filter) and frees it in feast_nh_destroy.
+ *  - The library allocates its workspace in feast_nh_init and frees it in
+ *    feast_nh_destroy.  One exception: banded shifted solves by inverted
+ *    diagonal blocks or by chunked tridiagonal recurrences, where a filter finds
+ *    that they do not reach opts.inner_tol, give their memory back in the middle
+ *    of that call and take the workspace of the triangular factors
+ *    instead.  The context keeps to those from then on.  The filter starts its
+ *    refinement again, up to opts.inner_max steps more; info->inner_steps counts
+ *    the steps of both.  If that workspace cannot be had the call returns
+ *    FEAST_NH_ENOMEM and a later one tries again.
  *  - Errors are returned, never raised or aborted; feast_nh_last_error gives
  *    a message for the last failing call on a context.  On FEAST_NH_ENOCONV
  *    the outputs hold the best iterate; on EINVAL/ECUDA they are undefined.
@@ -308,6 +315,9 @@ feast_nh_status feast_nh_release_memory(void);
 
 /* Device error-word bits, as reported through the status codes. */
 enum { FEAST_NH_DEVERR_ZERO_PIVOT = 1, FEAST_NH_DEVERR_QR_NOCONV = 2, FEAST_NH_DEVERR_TIMEOUT = 16 };
+/* A host-side bit of feast_nh_inject_device_error: the next workspace
+ * allocation on the context fails (FEAST_NH_ENOMEM). */
+enum { FEAST_NH_INJECT_NOMEM = 256 };
 
 /* Fault injection for tests, on the host: the next contour integration
  * (feast_nh_filter, or the first filter of feast_nh_solve) ORs `bits` into

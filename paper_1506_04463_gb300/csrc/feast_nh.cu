@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "feast_nh.h"
@@ -138,6 +139,7 @@ struct feast_nh_ctx {
   double *d_piv = nullptr;    // pivot statistics of the banded factors (2 doubles)
   double piv_min = 0, piv_max = 0;
   unsigned inject_bits = 0;   // host-requested device error bits (testing aid)
+  bool inject_nomem = false;  // the next workspace allocation fails (testing aid)
   bool rr_only = false;       // Rayleigh-Ritz workspace only (one problem of a batch)
   void *fgwork = nullptr;     // FGMRES workspace
   void *ework = nullptr;      // refined eigendecomposition workspace
@@ -181,7 +183,13 @@ P *dalloc(feast_nh_ctx *ctx, size_t bytes) {
   void *p = nullptr;
   if (bytes == 0) bytes = 16;
   bool pooled = false;
-  CKC(pool::alloc(&p, bytes, ctx->s, &pooled));
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (!std::exchange(ctx->inject_nomem, false)) e = pool::alloc(&p, bytes, ctx->s, &pooled);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here; not left for the next check of a launch
+    ctx->err = std::string("device workspace: ") + cudaGetErrorString(e);
+    throw Fail{e == cudaErrorMemoryAllocation ? FEAST_NH_ENOMEM : FEAST_NH_ECUDA};
+  }
   ctx->allocs.push_back(p);
   ctx->pooled.push_back(pooled);
   return reinterpret_cast<P *>(p);
@@ -311,15 +319,17 @@ void fg_precond(void *p, const cxf *v, cxf *z, cudaStream_t s) {
   }
 }
 
-// What the triangular solves need beside the factors: scratch and, in FP32
-// where the TMA form fits, room for the transposed factors, and tensor maps.
-void alloc_lu(feast_nh_ctx *ctx) {
+// What the triangular solves need beside the factors, as far as it is not
+// there yet: scratch and, in FP32 where the TMA form fits, room for the
+// transposed factors, and tensor maps.
+void ensure_lu(feast_nh_ctx *ctx) {
   const int n = ctx->n;
   const bool f32 = fp32(ctx);
   const size_t es = f32 ? sizeof(cxf) : sizeof(cxd);
-  ctx->ysc = dalloc<void>(ctx, es * (f32 ? band_solve_scratch_elems<float>(n, ctx->m0, ctx->ne)
-                                         : band_solve_scratch_elems<double>(n, ctx->m0, ctx->ne)));
-  if (f32 && band_tma_fits(ctx->klp, ctx->kup)) {
+  if (!ctx->ysc)
+    ctx->ysc = dalloc<void>(ctx, es * (f32 ? band_solve_scratch_elems<float>(n, ctx->m0, ctx->ne)
+                                           : band_solve_scratch_elems<double>(n, ctx->m0, ctx->ne)));
+  if (!ctx->bandT && f32 && band_tma_fits(ctx->klp, ctx->kup)) {
     ctx->bandT = dalloc<void>(ctx, (size_t)ctx->nf * n * (ctx->klp + ctx->kup + 1) * es);
     ctx->tma.assign(band_tma_bytes(), 0);
     if (!band_tma_make(ctx->tma.data(), n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band,
@@ -333,14 +343,23 @@ void transpose_lu(feast_nh_ctx *ctx) {
 }
 // The explicit inverses (or chunked recurrences) lose too much on this pencil:
 // their memory is given back, and this context keeps to the triangular factors.
+// If the memory of those cannot be had, the call ends with ENOMEM, and the next
+// one starts with the factorisation, which asks for it again.
 void leave_inverses(feast_nh_ctx *ctx) {
-  for (void **p : {&ctx->trico, &ctx->blkTc, &ctx->blkTr, &ctx->blkys}) {
+  ctx->factored = false;
+  BlockEntries &be = ctx->blkE;
+  for (void **p : {&ctx->trico, &ctx->blkTc, &ctx->blkTr, &ctx->blkys, &be.va[0], &be.va[1], &be.vb[0], &be.vb[1]}) {
     if (*p) dfree(ctx, *p);
     *p = nullptr;
   }
+  for (int *&p : be.idx) {
+    if (p) dfree(ctx, p);
+    p = nullptr;
+  }
   ctx->blk = ctx->tri = false;
-  alloc_lu(ctx);
+  ensure_lu(ctx);
   transpose_lu(ctx);
+  ctx->factored = true;
 }
 
 void factorize(feast_nh_ctx *ctx) {
@@ -349,6 +368,7 @@ void factorize(feast_nh_ctx *ctx) {
     ctx->t_factor = 0;
     return;
   }
+  if (!ctx->blk && !ctx->tri) ensure_lu(ctx);
   const CsrView *Bp = ctx->hasB ? &ctx->B : nullptr;
   CKC(cudaEventRecord(ctx->ev[4], ctx->s));
   CKC(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->s));
@@ -561,6 +581,7 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
       ctx->inner_steps = 1;
     }
     double last = 1.0;  // largest relative residual before the last solve
+    int before = 0;     // steps of solves given up for the triangular factors
     for (int it = 0; it < steps; ++it) {
       // residuals only: the node sum Q is formed once, from the final X
       int kr = ev_begin(ctx, ctx->ev_resid);
@@ -584,7 +605,7 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
       // one 8-byte read per refinement step decides whether to go on
       CKC(cudaMemcpyAsync(ctx->h_small, ctx->d_maxrel, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
       CKC(cudaStreamSynchronize(ctx->s));
-      ctx->inner_steps = it + 1;
+      ctx->inner_steps = before + it + 1;
       const double now = ctx->h_small[0];
       // FP64 solves by inverted blocks are refined once, which takes them to
       // the residual of the triangular factors
@@ -596,6 +617,7 @@ void do_filter(feast_nh_ctx *ctx, const cxd *Y, const cxd *Yh, cxd *Q, cxd *Qh, 
         leave_inverses(ctx);
         if (!(now < 1.0) || it + 1 >= steps) {
           first_solve();
+          before = it + 1;
           it = -1;
           continue;
         }
@@ -1020,7 +1042,7 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
         ctx->blk = hk <= kBlockMaxEntries;
         ctx->blkE.K = hk < 1 ? 1 : hk;
       }
-      if (!ctx->tri && !ctx->blk) alloc_lu(ctx);
+      if (!ctx->tri && !ctx->blk) ensure_lu(ctx);
       if (ctx->blk) {
         BlockEntries &be = ctx->blkE;
         const size_t cnt = block_entry_count(n, ctx->kl, ctx->ku, be.K);
@@ -1501,7 +1523,8 @@ feast_nh_status feast_nh_operator_loss(feast_nh_ctx *ctx, const float *out, cons
 
 feast_nh_status feast_nh_inject_device_error(feast_nh_ctx *ctx, uint32_t bits) {
   if (!ctx) return FEAST_NH_EINVAL;
-  ctx->inject_bits |= bits;
+  if (bits & FEAST_NH_INJECT_NOMEM) ctx->inject_nomem = true;
+  ctx->inject_bits |= bits & ~(uint32_t)FEAST_NH_INJECT_NOMEM;
   return FEAST_NH_OK;
 }
 

@@ -17,6 +17,7 @@ LIB_PATH = os.path.join(_HERE, "libfeast_nh.so")
 
 OK, EINVAL, ENOMEM, ECUDA, ENOCONV, EINNER, ESINGULAR, ETIMEOUT = range(8)
 DEVERR_ZERO_PIVOT, DEVERR_QR_NOCONV, DEVERR_TIMEOUT = 1, 2, 16
+INJECT_NOMEM = 256
 R64, C64 = 0, 1
 INNER_BANDED, INNER_BICGSTAB, INNER_FGMRES = 0, 1, 2
 PRECOND_NONE, PRECOND_JACOBI, PRECOND_LEARNED = 0, 1, 2

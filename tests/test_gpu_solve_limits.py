@@ -35,3 +35,33 @@ def test_more_blocks_than_a_grid_has_rows(prec):
         ref = sum((np.conj(wj) if side else wj) * f.solve(Y[side], trans="H" if side else "N") for f, wj in zip(lu, w))
         err = np.linalg.norm(out[side] - ref, axis=0)
         assert np.all(err <= (TOL + 1e-13) / 2.2 * np.linalg.norm(Y[side], axis=0)), (side, err.max())
+
+
+@pytest.mark.parametrize("prec", [F.PREC_FP32_IR, F.PREC_FP64])
+@pytest.mark.parametrize("bw", [1, 20])
+def test_no_memory_for_the_triangular_factors(prec, bw):
+    """A tolerance that nothing reaches sends a filter back to the triangular factors; their workspace fails.  The call
+    says so, and the next one asks for it again and gives the filter (||M^{-1}|| <= 1 as the bands below are diagonally
+    dominant: 8 - 5 - 2)."""
+    n, m = 200, 6
+    rng = np.random.default_rng(bw)
+    A = (sp.diags([rng.uniform(-1, 1, n - bw) for _ in range(2)], (-bw, bw)) + 8 * sp.eye(n)).tocsr()
+    con = wl.Contour(0, 4 + 0j, 1.0, ne=8)
+    Y = [rng.standard_normal((n, m)) + 1j * rng.standard_normal((n, m)) for _ in range(2)]
+    ctx = F.FeastNH(A, None, con, m, precision=prec, inner_tol=1e-30, inner_max=5)
+    out = [torch.empty((n, m), dtype=torch.complex128, device="cuda") for _ in range(2)]
+    blocks = [dev(y) for y in Y] + out
+    ptrs = [F._ptr(t) for t in blocks]
+    assert F.lib().feast_nh_inject_device_error(ctx.h, F.INJECT_NOMEM) == F.OK
+    assert F.lib().feast_nh_filter(ctx.h, *ptrs, m) == F.ENOMEM
+    z, w = F.nodes(con)
+    for _ in range(2):
+        assert F.lib().feast_nh_filter(ctx.h, *ptrs, m) == F.EINNER
+        for side in range(2):
+            ref = 0
+            for zj, wj in zip(z, w):
+                M = zj * np.eye(n) - A.toarray()
+                ref = ref + (np.conj(wj) * np.linalg.solve(M.conj().T, Y[1]) if side else wj * np.linalg.solve(M, Y[0]))
+            err = np.linalg.norm(host(out[side]) - ref, axis=0)
+            assert np.all(err <= 1e-12 * np.linalg.norm(Y[side], axis=0) * np.sum(np.abs(w)))
+    ctx.close()
