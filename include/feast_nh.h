@@ -313,6 +313,18 @@ feast_nh_status feast_nh_block_product(feast_nh_ctx *ctx, const void *X, const v
  * fails. */
 feast_nh_status feast_nh_release_memory(void);
 
+/* Fast forms that a general one stands behind, so that their failing shows in
+ * no result: which of them the context used.  TRIDIAGONAL, BLOCKS: its shifted
+ * solves are by chunked tridiagonal recurrences / inverted diagonal blocks (both
+ * clear: triangular factors, or a Krylov solver).  EIG_REFINED, NEAR_IDENTITY,
+ * ELIMINATION: the last small eigenproblem ended by refinement of its FP32 seed
+ * (else FP64 QR); the last B_U^{-1} was by Newton-Schulz steps (else
+ * Gauss-Jordan); the last B_Q was eliminated (else its eigendecomposition).
+ * For tests; waits for the stream. */
+enum { FEAST_NH_FORM_TRIDIAGONAL = 1, FEAST_NH_FORM_BLOCKS = 2, FEAST_NH_FORM_EIG_REFINED = 4,
+       FEAST_NH_FORM_ELIMINATION = 8, FEAST_NH_FORM_NEAR_IDENTITY = 16 };
+feast_nh_status feast_nh_forms(feast_nh_ctx *ctx, uint32_t *forms);
+
 /* Device error-word bits, as reported through the status codes. */
 enum { FEAST_NH_DEVERR_ZERO_PIVOT = 1, FEAST_NH_DEVERR_QR_NOCONV = 2, FEAST_NH_DEVERR_TIMEOUT = 16 };
 /* A host-side bit of feast_nh_inject_device_error: the next workspace

@@ -45,6 +45,7 @@ struct EigState {
   unsigned fmax[8];      // bits of max |F_ij| of each iteration
   double dsc[kMaxM0];    // D
   cxd d[2][kMaxM0];      // eigenvalues of M, ping-pong
+  int near;              // small_inv_near: the matrix was close to the identity
 };
 
 size_t small_eig_state_bytes() { return (sizeof(EigState) + 255) & ~(size_t)255; }
@@ -662,6 +663,7 @@ size_t small_eig_work_bytes() {
 }
 void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *Vinv, cxd *swork, void *work, int *d_err, cudaStream_t s) {
   if (m < 4) {  // one QR launch is shorter than the chain below (m = 3: 95 us against 120)
+    cudaMemsetAsync(work, 0, offsetof(EigState, dsc), s);
     small_eig_qr(A, m, lam, V, swork, d_err, nullptr, s);
     if (Vinv) small_inv(V, m, Vinv, swork, d_err, nullptr, s);
     return;
@@ -762,14 +764,21 @@ void small_inv_near(const cxd *B, int m, cxd *Binv, cxd *swork, void *work, int 
   cxd *b = reinterpret_cast<cxd *>(reinterpret_cast<unsigned char *>(work) + small_eig_state_bytes());
   const size_t mm = (size_t)m * m;
   cxd *X0 = b, *C = b + mm, *X1 = b + 2 * mm;
-  k_inv_start<<<1, 512, 0, s>>>(m, B, X0, &st->done);
+  k_inv_start<<<1, 512, 0, s>>>(m, B, X0, &st->near);
   note_launch();
-  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, B, X0, C, 0, &st->done);
-  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, X0, C, X1, 1, &st->done);
-  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, B, X1, C, 0, &st->done);
-  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, X1, C, Binv, 1, &st->done);
+  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, B, X0, C, 0, &st->near);
+  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, X0, C, X1, 1, &st->near);
+  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, B, X1, C, 0, &st->near);
+  k_inv_step<<<tile_grid(m), 128, 0, s>>>(m, X1, C, Binv, 1, &st->near);
   for (int k = 0; k < 4; ++k) note_launch();
-  small_inv(B, m, Binv, swork, d_err, &st->done, s);
+  small_inv(B, m, Binv, swork, d_err, &st->near, s);
+}
+
+cudaError_t small_forms(const void *work, int *refined, int *near, cudaStream_t s) {
+  const EigState *st = reinterpret_cast<const EigState *>(work);
+  cudaError_t e = cudaMemcpyAsync(refined, &st->done, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(near, &st->near, sizeof(int), cudaMemcpyDeviceToHost, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
 }
 
 // Complex symmetric reduced problem (Sec. 2.4): W scaled so that w^T B_U w = 1,

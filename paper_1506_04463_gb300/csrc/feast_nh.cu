@@ -1124,6 +1124,7 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     ctx->Wh = dalloc<cxd>(ctx, sm);
     ctx->swork = dalloc<cxd>(ctx, 3 * sm);
     ctx->ework = dalloc<void>(ctx, small_eig_work_bytes());
+    CKC(cudaMemsetAsync(ctx->ework, 0, small_eig_work_bytes(), ctx->s));
     ctx->gchunks = gram_chunks(n);
     ctx->gpart = dalloc<cxd>(ctx, std::max((size_t)ctx->gchunks * sm, gram_tc_part_max(n)));
     ctx->d_fxy = dalloc<int>(ctx, 2 * kMaxM0 * sizeof(int));
@@ -1147,6 +1148,7 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     ctx->sxh = dalloc<cxd>(ctx, kMaxM0 * sizeof(cxd));
     CKC(cudaMemsetAsync(ctx->d_st, 0, sizeof(RRStatus), ctx->s));
     CKC(cudaMallocHost((void **)&ctx->h_st, sizeof(RRStatus)));
+    *ctx->h_st = RRStatus{};
     CKC(cudaMallocHost((void **)&ctx->h_small, 4 * sizeof(double)));
     CKC(cudaStreamSynchronize(ctx->s));
     check_launch(ctx, "init");
@@ -1518,6 +1520,20 @@ feast_nh_status feast_nh_operator_loss(feast_nh_ctx *ctx, const float *out, cons
   } catch (const Fail &f) {
     return f.st;
   }
+  return FEAST_NH_OK;
+}
+
+feast_nh_status feast_nh_forms(feast_nh_ctx *ctx, uint32_t *forms) {
+  if (!ctx || !forms) return FEAST_NH_EINVAL;
+  int refined = 0, near = 0;
+  try {
+    CKC(small_forms(ctx->ework, &refined, &near, ctx->s));
+  } catch (const Fail &f) {
+    return f.st;
+  }
+  *forms = (ctx->tri ? FEAST_NH_FORM_TRIDIAGONAL : 0) | (ctx->blk ? FEAST_NH_FORM_BLOCKS : 0) |
+           (refined ? FEAST_NH_FORM_EIG_REFINED : 0) | (ctx->h_st->biorth ? FEAST_NH_FORM_ELIMINATION : 0) |
+           (near ? FEAST_NH_FORM_NEAR_IDENTITY : 0);
   return FEAST_NH_OK;
 }
 

@@ -270,5 +270,8 @@ size_t small_eig_work_bytes();
 void small_eig(const cxd *A, int m, cxd *lam, cxd *V, cxd *Vinv, cxd *swork, void *work, int *d_err, cudaStream_t s);
 // Inverse of a matrix that is usually within 1e-3 of the identity.
 void small_inv_near(const cxd *B, int m, cxd *Binv, cxd *swork, void *work, int *d_err, cudaStream_t s);
+// Whether the last small_eig ended by refinement, and the last small_inv_near by
+// Newton-Schulz steps, on this workspace (zeroed before its first use).
+cudaError_t small_forms(const void *work, int *refined, int *near, cudaStream_t s);
 // C = A B, or (A B)^H with herm.
 void small_prod(int m, const cxd *A, const cxd *B, cxd *C, int herm, cudaStream_t s);

@@ -18,6 +18,7 @@ LIB_PATH = os.path.join(_HERE, "libfeast_nh.so")
 OK, EINVAL, ENOMEM, ECUDA, ENOCONV, EINNER, ESINGULAR, ETIMEOUT = range(8)
 DEVERR_ZERO_PIVOT, DEVERR_QR_NOCONV, DEVERR_TIMEOUT = 1, 2, 16
 INJECT_NOMEM = 256
+FORM_TRIDIAGONAL, FORM_BLOCKS, FORM_EIG_REFINED, FORM_ELIMINATION, FORM_NEAR_IDENTITY = 1, 2, 4, 8, 16
 R64, C64 = 0, 1
 INNER_BANDED, INNER_BICGSTAB, INNER_FGMRES = 0, 1, 2
 PRECOND_NONE, PRECOND_JACOBI, PRECOND_LEARNED = 0, 1, 2
@@ -73,7 +74,7 @@ class BatchInfo(C.Structure):
 EXPORTS = ["feast_nh_default_opts", "feast_nh_init", "feast_nh_filter", "feast_nh_rr", "feast_nh_solve",
            "feast_nh_destroy", "feast_nh_strerror", "feast_nh_last_error", "feast_nh_nodes",
            "feast_nh_multishift_residual", "feast_nh_kernel_launches", "feast_nh_multishift_residual_noalloc",
-           "feast_nh_small_eig", "feast_nh_inject_device_error", "feast_nh_batch_init", "feast_nh_batch_solve",
+           "feast_nh_small_eig", "feast_nh_forms", "feast_nh_inject_device_error", "feast_nh_batch_init", "feast_nh_batch_solve",
            "feast_nh_batch_destroy", "feast_nh_batch_last_error", "feast_nh_multishift_spmm", "feast_nh_net_create",
            "feast_nh_net_set_params", "feast_nh_net_get_params", "feast_nh_net_forward", "feast_nh_net_train_step",
            "feast_nh_net_destroy", "feast_nh_net_last_error", "feast_nh_set_network", "feast_nh_learned_pairs",
@@ -114,6 +115,8 @@ def lib():
     L.feast_nh_block_product.argtypes = [vp, vp, vp, i32, i32, vp, i32]
     L.feast_nh_multishift_spmm.argtypes = [vp, vp, vp, i32, i32]
     L.feast_nh_inject_device_error.argtypes = [vp, C.c_uint32]
+    L.feast_nh_forms.argtypes = [vp, C.POINTER(C.c_uint32)]
+    L.feast_nh_forms.restype = i32
     L.feast_nh_multishift_residual_noalloc.argtypes = [C.POINTER(Csr), C.POINTER(Csr), C.POINTER(ContourS), vp, vp,
                                                        vp, vp, vp, i32, vp]
     L.feast_nh_multishift_residual_noalloc.restype = i32
@@ -442,6 +445,12 @@ class FeastNH:
         st = lib().feast_nh_set_network(self.h, net.h, int(N), float(kappa),
                                         f.ctypes.data_as(C.POINTER(C.c_float)) if f.size else None, int(f.size))
         self._check(st, "feast_nh_set_network")
+
+    def forms(self) -> int:
+        """FORM_* bits: the fast forms this context used last (tests)."""
+        v = C.c_uint32()
+        self._check(lib().feast_nh_forms(self.h, C.byref(v)), "feast_nh_forms")
+        return v.value
 
     def inject_device_error(self, bits):
         """Host-side fault injection: the next filter ORs `bits` into the
