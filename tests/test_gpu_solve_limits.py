@@ -65,3 +65,42 @@ def test_no_memory_for_the_triangular_factors(prec, bw):
             err = np.linalg.norm(host(out[side]) - ref, axis=0)
             assert np.all(err <= 1e-12 * np.linalg.norm(Y[side], axis=0) * np.sum(np.abs(w)))
     ctx.close()
+
+
+
+@pytest.mark.parametrize("inner_max", [1, 12])
+def test_tridiagonal_fp64_residual(inner_max):
+    """Three pivots of 1e-5, so that the chunked recurrences alone leave a residual of 5e-13 to 2e-12 (emulated in
+    numpy): below inner_tol, but far above a refined solve's, eps (|M| |x| + |y|) / |y| = 1e-15 here.  One node with
+    weight one: Q is the solution itself.  With a single step the triangular factors are taken, whose growth by the
+    small pivots is eps / 1e-5."""
+    n, m = 500, 3
+    rng = np.random.default_rng(2)
+    lo, up, di = rng.uniform(0.5, 1, n), rng.uniform(0.5, 1, n), 4 + rng.uniform(0, 1, n)
+    d = di[0]
+    for r in range(1, n):
+        d = di[r] - lo[r] / d * up[r - 1]
+        if r in (100, 250, 400):
+            di[r] += 1e-5 - d
+            d = 1e-5
+    A = sp.diags([lo[1:], di, up[:-1]], [-1, 0, 1]).tocsr()
+    con = wl.Contour(2, 0j, 1.0, z=np.array([0j]), w=np.array([1 + 0j]))
+    Y = [rng.standard_normal((n, m)) + 1j * rng.standard_normal((n, m)) for _ in range(2)]
+    ctx = F.FeastNH(A, None, con, m, precision=F.PREC_FP64, inner_tol=TOL, inner_max=inner_max)
+    Q = [host(t) for t in ctx.filter(*(dev(y) for y in Y))]
+    assert bool(ctx.forms() & F.FORM_TRIDIAGONAL) == (inner_max > 1)
+    ctx.close()
+    for C, y, q in zip((A, A.T), Y, Q):
+        res = np.linalg.norm(y + C @ q, axis=0) / np.linalg.norm(y, axis=0)
+        assert np.all(res <= (5e-15 if inner_max > 1 else 2.3e-11)), res
+
+
+def test_single_step_fp64_blocks():
+    """No step left to refine solves by inverted blocks: triangular factors."""
+    n, m = 200, 4
+    rng = np.random.default_rng(3)
+    A = (sp.diags([rng.uniform(-1, 1, n - 20) for _ in range(2)], (-20, 20)) + 8 * sp.eye(n)).tocsr()
+    ctx = F.FeastNH(A, None, wl.Contour(0, 4 + 0j, 1.0, ne=4), m, precision=F.PREC_FP64, inner_tol=TOL, inner_max=1)
+    ctx.filter(*(dev(rng.standard_normal((n, m))) for _ in range(2)))
+    assert ctx.forms() & (F.FORM_TRIDIAGONAL | F.FORM_BLOCKS) == 0
+    ctx.close()
