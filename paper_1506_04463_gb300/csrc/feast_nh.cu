@@ -61,6 +61,20 @@ cudaError_t alloc(void **ptr, size_t bytes, cudaStream_t s, bool *pooled) {
   *pooled = mp != nullptr;
   return mp ? cudaMallocFromPoolAsync(ptr, bytes, mp, s) : cudaMalloc(ptr, bytes);
 }
+// Device memory that an allocation can still get: free, or reserved by the pool and unused.
+size_t available() {
+  size_t free_b = 0, total = 0;
+  uint64_t reserved = 0, used = 0;
+  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cudaMemPool_t mp = get();
+  if (mp && cudaMemPoolGetAttribute(mp, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+      cudaMemPoolGetAttribute(mp, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+    free_b += reserved - used;
+  return free_b;
+}
 void release(void *ptr, bool pooled, cudaStream_t s) {
   if (pooled)
     cudaFreeAsync(ptr, s);
@@ -341,12 +355,8 @@ void transpose_lu(feast_nh_ctx *ctx) {
   if (!ctx->tma.empty())
     launch_band_transpose(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxf *)ctx->band, (cxf *)ctx->bandT, ctx->s);
 }
-// The explicit inverses (or chunked recurrences) lose too much on this pencil:
-// their memory is given back, and this context keeps to the triangular factors.
-// If the memory of those cannot be had, the call ends with ENOMEM, and the next
-// one starts with the factorisation, which asks for it again.
-void leave_inverses(feast_nh_ctx *ctx) {
-  ctx->factored = false;
+// The solves by inverted blocks or chunked recurrences given up, and their memory.
+void free_inverses(feast_nh_ctx *ctx) {
   BlockEntries &be = ctx->blkE;
   for (void **p : {&ctx->trico, &ctx->blkTc, &ctx->blkTr, &ctx->blkys, &be.va[0], &be.va[1], &be.vb[0], &be.vb[1]}) {
     if (*p) dfree(ctx, *p);
@@ -357,9 +367,80 @@ void leave_inverses(feast_nh_ctx *ctx) {
     p = nullptr;
   }
   ctx->blk = ctx->tri = false;
+}
+// The explicit inverses (or chunked recurrences) lose too much on this pencil:
+// their memory is given back, and this context keeps to the triangular factors.
+// If the memory of those cannot be had, the call ends with ENOMEM, and the next
+// one starts with the factorisation, which asks for it again.
+void leave_inverses(feast_nh_ctx *ctx) {
+  ctx->factored = false;
+  free_inverses(ctx);
   ensure_lu(ctx);
   transpose_lu(ctx);
   ctx->factored = true;
+}
+// Memory of the solves by inverted blocks or chunked recurrences (ctx->blk,
+// ctx->tri chosen).  The two copies of the inverses take as much as the band
+// itself (in FP32 they come in place of bandT, in FP64 on top of all else), for
+// bands narrower than a block of 16 more.  They must not make a pencil too large
+// that fits with the triangular factors: called last, allowed half of what those
+// would leave available, and given up where that does not do.
+void alloc_inverses(feast_nh_ctx *ctx) {
+  const int n = ctx->n, m0 = ctx->m0, ne = ctx->ne, nf = ctx->nf;
+  const bool f32 = fp32(ctx);
+  const size_t es = f32 ? sizeof(cxf) : sizeof(cxd);
+  const size_t tri_co = tri_elems(n, nf) * es, inv = block_elems(n, ctx->kl, ctx->ku, nf) * es;
+  // FP64: also room for the 16 x 16 inverses that the blocks' are formed from
+  const size_t ys = ctx->tri ? tri_scratch_elems(n, m0, ne) * es
+                             : std::max(block_scratch_elems(n, ctx->kl, ctx->ku, m0, ne),
+                                        f32 ? 0 : band_diag_inv_elems(n, nf)) * es;
+  const size_t extra = ctx->tri ? tri_co + ys : 2 * inv + ys;
+  const size_t lu = es * (f32 ? band_solve_scratch_elems<float>(n, m0, ne) : band_solve_scratch_elems<double>(n, m0, ne)) +
+                    (f32 && band_tma_fits(ctx->klp, ctx->kup) ? (size_t)nf * n * (ctx->klp + ctx->kup + 1) * es : 0);
+  try {
+    if (extra > lu + (256u << 20)) {  // not asked for less: the answer takes 0.3 ms
+      const size_t avail = pool::available();
+      if (extra > lu + (avail > lu ? (avail - lu) / 2 : 0)) throw Fail{FEAST_NH_ENOMEM};
+    }
+    if (ctx->tri) ctx->trico = dalloc<void>(ctx, tri_co);
+    ctx->blkys = dalloc<void>(ctx, ys);
+    if (ctx->blk) {
+      ctx->blkTc = dalloc<void>(ctx, inv);
+      ctx->blkTr = dalloc<void>(ctx, inv);
+    }
+  } catch (const Fail &f) {
+    if (f.st != FEAST_NH_ENOMEM) throw;
+    ctx->err.clear();
+    free_inverses(ctx);
+    ensure_lu(ctx);
+  }
+}
+// The off-diagonal entries of the block form, both sides; without room for them
+// the triangular factors.
+void form_entries(feast_nh_ctx *ctx) {
+  const bool f32 = fp32(ctx);
+  const size_t es = f32 ? sizeof(cxf) : sizeof(cxd);
+  BlockEntries &be = ctx->blkE;
+  const size_t cnt = block_entry_count(ctx->n, ctx->kl, ctx->ku, be.K);
+  try {
+    for (int k = 0; k < 2; ++k) {
+      be.idx[k] = dalloc<int>(ctx, cnt * sizeof(int));
+      be.va[k] = dalloc<void>(ctx, cnt * es);
+      be.vb[k] = ctx->hasB ? dalloc<void>(ctx, cnt * es) : nullptr;
+    }
+  } catch (const Fail &f) {
+    if (f.st != FEAST_NH_ENOMEM) throw;
+    ctx->err.clear();
+    free_inverses(ctx);
+    return;
+  }
+  for (int k = 0; k < 2; ++k) {
+    const CsrView &M = k ? ctx->AH : ctx->A, *N = ctx->hasB ? (k ? &ctx->BH : &ctx->B) : nullptr;
+    if (f32)
+      launch_block_entries<float>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxf *)be.va[k], (cxf *)be.vb[k], ctx->s);
+    else
+      launch_block_entries<double>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxd *)be.va[k], (cxd *)be.vb[k], ctx->s);
+  }
 }
 
 void factorize(feast_nh_ctx *ctx) {
@@ -387,10 +468,11 @@ void factorize(feast_nh_ctx *ctx) {
     if (ctx->tri) {
       launch_tri_setup<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band, (cxd *)ctx->trico, ctx->s);
     } else if (ctx->blk) {
-      launch_band_diag_inv<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band, (cxd *)ctx->dinv,
+      // the 16 x 16 inverses are only an intermediate here: in the solves' scratch
+      launch_band_diag_inv<double>(ctx->n, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band, (cxd *)ctx->blkys,
                                    ctx->s);
       CKC(block_invert<double>(ctx->n, ctx->kl, ctx->ku, ctx->klp, ctx->kup, ctx->nf, (const cxd *)ctx->band,
-                               (const cxd *)ctx->dinv, (cxd *)ctx->blkTc, (cxd *)ctx->blkTr, ctx->s));
+                               (const cxd *)ctx->blkys, (cxd *)ctx->blkTc, (cxd *)ctx->blkTr, ctx->s));
     }
   }
   if (!ctx->blk && !ctx->tri) transpose_lu(ctx);
@@ -1041,10 +1123,6 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
       // the triangular factors, so that opts have to allow one
       const bool room = f32 || ctx->o.inner_max > 1;
       ctx->tri = room && ctx->kl <= 1 && ctx->ku <= 1;
-      if (ctx->tri) {
-        ctx->trico = dalloc<void>(ctx, tri_elems(n, ctx->nf) * es);
-        ctx->blkys = dalloc<void>(ctx, tri_scratch_elems(n, m0, ne) * es);
-      }
       if (room && !ctx->tri && block_solve_fits(ctx->kl, ctx->ku)) {
         // off-diagonal entries of a row between blocks, both sides
         int *d_k = dalloc<int>(ctx, sizeof(int)), hk = 0;
@@ -1056,29 +1134,9 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
         ctx->blk = hk <= kBlockMaxEntries;
         ctx->blkE.K = hk < 1 ? 1 : hk;
       }
+      if (ctx->blk) form_entries(ctx);
       if (!ctx->tri && !ctx->blk) ensure_lu(ctx);
-      if (ctx->blk) {
-        BlockEntries &be = ctx->blkE;
-        const size_t cnt = block_entry_count(n, ctx->kl, ctx->ku, be.K);
-        for (int k = 0; k < 2; ++k) {
-          const CsrView &M = k ? ctx->AH : ctx->A, *N = B ? (k ? &ctx->BH : &ctx->B) : nullptr;
-          be.idx[k] = dalloc<int>(ctx, cnt * sizeof(int));
-          be.va[k] = dalloc<void>(ctx, cnt * es);
-          be.vb[k] = B ? dalloc<void>(ctx, cnt * es) : nullptr;
-          if (f32)
-            launch_block_entries<float>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxf *)be.va[k], (cxf *)be.vb[k],
-                                        ctx->s);
-          else
-            launch_block_entries<double>(M, N, ctx->kl, ctx->ku, be.K, be.idx[k], (cxd *)be.va[k], (cxd *)be.vb[k],
-                                         ctx->s);
-        }
-      }
-      if (f32 || ctx->blk) ctx->dinv = dalloc<void>(ctx, band_diag_inv_elems(n, ctx->nf) * es);
-      if (ctx->blk) {
-        ctx->blkTc = dalloc<void>(ctx, block_elems(n, ctx->kl, ctx->ku, ctx->nf) * es);
-        ctx->blkTr = dalloc<void>(ctx, block_elems(n, ctx->kl, ctx->ku, ctx->nf) * es);
-        ctx->blkys = dalloc<void>(ctx, block_scratch_elems(n, ctx->kl, ctx->ku, m0, ne) * es);
-      }
+      if (f32) ctx->dinv = dalloc<void>(ctx, band_diag_inv_elems(n, ctx->nf) * es);
     }
     if (inner && fgmres(ctx)) {
       ctx->fgwork = dalloc<void>(ctx, fgmres_work_bytes(n, m0, ne, ctx->o.krylov_restart));
@@ -1161,6 +1219,7 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     ctx->sx = dalloc<cxd>(ctx, kMaxM0 * sizeof(cxd));
     ctx->sxh = dalloc<cxd>(ctx, kMaxM0 * sizeof(cxd));
     CKC(cudaMemsetAsync(ctx->d_st, 0, sizeof(RRStatus), ctx->s));
+    if (ctx->tri || ctx->blk) alloc_inverses(ctx);
     CKC(cudaMallocHost((void **)&ctx->h_st, sizeof(RRStatus)));
     *ctx->h_st = RRStatus{};
     CKC(cudaMallocHost((void **)&ctx->h_small, 4 * sizeof(double)));

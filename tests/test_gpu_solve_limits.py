@@ -104,3 +104,40 @@ def test_single_step_fp64_blocks():
     ctx.filter(*(dev(rng.standard_normal((n, m))) for _ in range(2)))
     assert ctx.forms() & (F.FORM_TRIDIAGONAL | F.FORM_BLOCKS) == 0
     ctx.close()
+
+
+def test_no_room_for_the_inverses():
+    """Memory for the factors and all other workspace, but not for the inverted blocks: the context is created all the
+    same, with the triangular factors, and filters like one that has them (both to TOL; ||M^{-1}|| <= 1 / (8 - 5 - 2),
+    the sum of the weights' moduli is 1).  In FP64 they come on top of all that the triangular factors need."""
+    n, m, bw, ne = 40000, 4, 64, 8
+    rng = np.random.default_rng(9)
+    A = (sp.diags([rng.uniform(-1, 1, n - bw) for _ in range(2)], (-bw, bw)) + (8 + 0j) * sp.eye(n)).tocsr()
+    con = wl.Contour(0, 4 + 0j, 1.0, ne=ne)
+    Y = [dev(rng.standard_normal((n, m))) for _ in range(2)]
+    inverse = ne * n * bw * 16  # one of the two copies
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        F.release_memory()
+        return torch.cuda.mem_get_info()[0]
+
+    before = free()
+    ctx = F.FeastNH(A, None, con, m, precision=F.PREC_FP64, inner_tol=TOL)
+    assert ctx.forms() & F.FORM_BLOCKS
+    ref = [host(q) for q in ctx.filter(*Y)]
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    ctx.close()
+    filler = torch.empty(free() - (used - inverse), dtype=torch.uint8, device="cuda")
+    try:
+        ctx = F.FeastNH(A, None, con, m, precision=F.PREC_FP64, inner_tol=TOL)
+        assert ctx.forms() & F.FORM_BLOCKS == 0
+        out = [host(q) for q in ctx.filter(*Y)]
+        ctx.close()
+    finally:
+        del filler
+        free()
+    for a, b, y in zip(out, ref, Y):
+        assert np.all(np.linalg.norm(a - b, axis=0) <= 2 * (TOL + 1e-13) * np.linalg.norm(host(y), axis=0))
