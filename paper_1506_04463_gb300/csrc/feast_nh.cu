@@ -104,6 +104,7 @@ struct feast_nh_ctx {
   std::vector<void *> allocs;
   std::vector<bool> pooled;  // allocs[i] came from the library's pool
   int kl = -1, ku = -1;     // band of (z B - A)
+  int longest[2] = {0, 0};  // entries of the longest row of A and of A^H
   int klp = 0, kup = 0;     // stored band widths (kl rounded up to even, kl+ku+1 even)
   void *bandT = nullptr;    // FP32: transposed factors for the conjugate-transpose solves
   void *kwork = nullptr;    // BiCGStab workspace
@@ -310,11 +311,11 @@ void fg_apply(void *p, const cxf *x, cxf *y, cudaStream_t s) {
   const FgSide *f = static_cast<const FgSide *>(p);
   feast_nh_ctx *ctx = f->ctx;
   if (f->side == 0)
-    launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 0, x, y,
-                               f->m, s);
+    launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->longest[0],
+                               ctx->ne, ctx->dz, 0, x, y, f->m, s);
   else
-    launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 1, x, y,
-                               f->m, s);
+    launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->longest[1],
+                               ctx->ne, ctx->dz, 1, x, y, f->m, s);
 }
 void fg_precond(void *p, const cxf *v, cxf *z, cudaStream_t s) {
   const FgSide *f = static_cast<const FgSide *>(p);
@@ -1223,6 +1224,10 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
     CKC(cudaMallocHost((void **)&ctx->h_st, sizeof(RRStatus)));
     *ctx->h_st = RRStatus{};
     CKC(cudaMallocHost((void **)&ctx->h_small, 4 * sizeof(double)));
+    if (inner) {
+      launch_longest_rows(ctx->A, ctx->AH, ctx->d_ext, ctx->s);
+      CKC(cudaMemcpyAsync(ctx->longest, ctx->d_ext, 2 * sizeof(int), cudaMemcpyDeviceToHost, ctx->s));
+    }
     CKC(cudaStreamSynchronize(ctx->s));
     check_launch(ctx, "init");
   }
@@ -1442,11 +1447,11 @@ feast_nh_status feast_nh_multishift_spmm(feast_nh_ctx *ctx, const void *P, void 
     REQ(P && V && m >= 1 && m <= ctx->m0 && (side == 0 || side == 1), "multishift_spmm: bad arguments");
     REQ(!ctx->rr_only, "multishift_spmm: context has no operator");
     if (side == 0)
-      launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 0,
-                                 (const cxf *)P, (cxf *)V, m, ctx->s);
+      launch_multishift_spmm_f32(ctx->A, ctx->hasB ? &ctx->B : nullptr, ctx->kl + ctx->ku + 1, ctx->longest[0],
+                                 ctx->ne, ctx->dz, 0, (const cxf *)P, (cxf *)V, m, ctx->s);
     else
-      launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->ne, ctx->dz, 1,
-                                 (const cxf *)P, (cxf *)V, m, ctx->s);
+      launch_multishift_spmm_f32(ctx->AH, ctx->hasB ? &ctx->BH : nullptr, ctx->kl + ctx->ku + 1, ctx->longest[1],
+                                 ctx->ne, ctx->dz, 1, (const cxf *)P, (cxf *)V, m, ctx->s);
     check_launch(ctx, "multishift_spmm");
   } catch (const Fail &f) {
     return f.st;

@@ -108,10 +108,12 @@ int launch_multishift_residual_capped(const CsrView &A, const CsrView *B, int ne
 void launch_residual_check(const double *partial, int nparts, int ne, int m, const double *bynorm2, int nsides,
                            double *d_maxrel, cudaStream_t s);
 // FP32 multi-shift operator V_j = (z_j B - A) P_j (conj_z: conj(z_j), for the
-// conjugate-transpose CSR pair) over node-major complex-float blocks; returns
-// the grid needed for one row group a warp.  bw: width of the pencil's band.
-int launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z,
-                               const cxf *P, cxf *V, int m, cudaStream_t s);
+// conjugate-transpose CSR pair) over node-major complex-float blocks.  bw:
+// width of the pencil's band; longest: entries of A's longest row.
+void launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int longest, int ne, const cxd *d_z,
+                                int conj_z, const cxf *P, cxf *V, int m, cudaStream_t s);
+// Longest row of A [0] and of A^H [1] (entries).
+void launch_longest_rows(const CsrView &A, const CsrView &AH, int *d_out, cudaStream_t s);
 // Out = M1 X - shift_c (M2 X)  (M2 == NULL: identity), row-major n x m blocks.
 // If p1/p2 != NULL, per-CTA partial column 1-norms of Out and of (M2 X).
 int launch_spmm(const CsrView &M1, const CsrView *M2, const cxd *shift, const cxd *X, cxd *Out, int m,

@@ -671,15 +671,29 @@ __global__ void __launch_bounds__(kSpThreads, U == 5 ? 4 : PAIR ? 3 : 2)
 }
 
 
-// Rows of up to five entries, more than 32 columns (even), no B, all nodes at
-// once: a warp a row, whose entries every lane reads itself.  16 nodes, 64
-// columns of the 300 x 300 grid 291 us and 48 columns, 8 nodes 144 us, against
-// 320 and 162 with the lanes' entries above; longer rows take the loop.
-template <bool ACPLX>
+// VW columns of a lane: neighbours (VW = 2, rows start on 16 bytes) or one.
+template <int VW> __device__ __forceinline__ float4 loadw(const cxf *p) {
+  if constexpr (VW == 2) return *reinterpret_cast<const float4 *>(p);
+  const float2 a = *reinterpret_cast<const float2 *>(p);
+  return make_float4(a.x, a.y, 0.f, 0.f);
+}
+template <int VW> __device__ __forceinline__ void storew(cxf *p, float4 v) {
+  if constexpr (VW == 2)
+    *reinterpret_cast<float4 *>(p) = v;
+  else
+    *reinterpret_cast<float2 *>(p) = make_float2(v.x, v.y);
+}
+
+// More than 32 columns, no B, rows of up to K entries (longer ones take a
+// loop): a warp a row, whose entries every lane reads and keeps itself, for ng
+// nodes at a time.  Bound by the gathers out of L2, K + 1 in flight
+// a lane; the group kernel above spends as many issue slots on its shuffles,
+// and past nine entries it has no row in registers.  What each K measured
+// against it stands with the rule below.
+template <bool ACPLX, int VW, int K>
 __global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView A, int ne, const cxd *__restrict__ z,
                                                                          int conj_z, const cxf *__restrict__ P,
-                                                                         cxf *__restrict__ V, int n, int m) {
-  constexpr int K = 5;
+                                                                         cxf *__restrict__ V, int n, int m, int ng) {
   __shared__ cxf zs[kMaxNe];
   if (threadIdx.x < ne) {
     const cxd zz = z[threadIdx.x];
@@ -690,64 +704,74 @@ __global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView
   const int warp = (int)(((long long)blockIdx.x * kSpThreads + threadIdx.x) >> 5);
   const int nwarps = (int)(((long long)gridDim.x * kSpThreads) >> 5);
   const size_t xns = (size_t)n * m;
-  auto entry = [&](int64_t k) {  // of A
+  auto entry = [&](int64_t k) {  // of -A
     if constexpr (ACPLX) {
       const cxd v = reinterpret_cast<const cxd *>(A.val)[k];
-      return mk((float)v.re, A.conj_vals ? -(float)v.im : (float)v.im);
+      return mk(-(float)v.re, A.conj_vals ? (float)v.im : -(float)v.im);
     }
-    return mk((float)A.val[k], 0.f);
+    return mk(-(float)A.val[k], 0.f);
   };
-  auto sub = [](float4 &acc, cxf a, const float4 &x) {  // acc -= a x
-    acc.x = fmaf(-a.re, x.x, acc.x);
-    acc.x = fmaf(a.im, x.y, acc.x);
-    acc.y = fmaf(-a.re, x.y, acc.y);
-    acc.y = fmaf(-a.im, x.x, acc.y);
-    acc.z = fmaf(-a.re, x.z, acc.z);
-    acc.z = fmaf(a.im, x.w, acc.z);
-    acc.w = fmaf(-a.re, x.w, acc.w);
-    acc.w = fmaf(-a.im, x.z, acc.w);
-  };
-  for (int i = warp; i < n; i += nwarps) {
-    const int64_t ka = A.rowptr[i];
-    const int nk = (int)(A.rowptr[i + 1] - ka);
-    int col[K];
-    cxf av[K];
+  for (int j0 = 0; j0 < ne; j0 += ng) {
+    const int j1 = min(ne, j0 + ng);
+    for (int i = warp; i < n; i += nwarps) {
+      const int64_t ka = A.rowptr[i];
+      const int nk = (int)(A.rowptr[i + 1] - ka);
+      int col[K];
+      cxf av[K];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      col[k] = k < nk ? A.colind[ka + k] : i;
-      av[k] = k < nk ? entry(ka + k) : mk(0.f, 0.f);
-    }
-    const bool fast = nk <= K;
-    for (int c = lane * 2; c < m; c += 64) {
+      for (int k = 0; k < K; ++k) {
+        col[k] = k < nk ? A.colind[ka + k] : i;
+        av[k] = k < nk ? entry(ka + k) : mk(0.f, 0.f);
+      }
+      const bool fast = nk <= K;
+      for (int c = lane * VW; c < m; c += 32 * VW) {
 #pragma unroll 2
-      for (int j = 0; j < ne; ++j) {
-        const cxf *Pj = P + (size_t)j * xns;
-        float4 acc;
-        acc.x = acc.y = 0.f;
-        acc.z = acc.w = 0.f;
-        if (fast) {
-          float4 xs[K];
+        for (int j = j0; j < j1; ++j) {
+          const cxf *Pj = P + (size_t)j * xns + c;
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (fast) {
+            float4 xs[K];
 #pragma unroll
-          for (int k = 0; k < K; ++k) xs[k] = *reinterpret_cast<const float4 *>(Pj + (size_t)col[k] * m + c);
-          vfma<true>(acc, zs[j], *reinterpret_cast<const float4 *>(Pj + (size_t)i * m + c));
+            for (int k = 0; k < K; ++k) xs[k] = loadw<VW>(Pj + (size_t)col[k] * m);
+            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m));
 #pragma unroll
-          for (int k = 0; k < K; ++k) sub(acc, av[k], xs[k]);
-        } else {
-          vfma<true>(acc, zs[j], *reinterpret_cast<const float4 *>(Pj + (size_t)i * m + c));
-          for (int k = 0; k < nk; ++k)
-            sub(acc, entry(ka + k), *reinterpret_cast<const float4 *>(Pj + (size_t)A.colind[ka + k] * m + c));
+            for (int k = 0; k < K; ++k) vfma<ACPLX>(acc, av[k], xs[k]);
+          } else {
+            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m));
+            for (int k = 0; k < nk; ++k)
+              vfma<ACPLX>(acc, entry(ka + k), loadw<VW>(Pj + (size_t)A.colind[ka + k] * m));
+          }
+          storew<VW>(V + (size_t)j * xns + (size_t)i * m + c, acc);
         }
-        *reinterpret_cast<float4 *>(V + (size_t)j * xns + (size_t)i * m + c) = acc;
       }
     }
   }
 }
 
+// Longest row of A and of A^H.
+__global__ void k_longest_rows(CsrView A, CsrView AH, int *out) {
+  int mx[2] = {0, 0};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += gridDim.x * blockDim.x) {
+    mx[0] = max(mx[0], (int)(A.rowptr[i + 1] - A.rowptr[i]));
+    mx[1] = max(mx[1], (int)(AH.rowptr[i + 1] - AH.rowptr[i]));
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int v = __reduce_max_sync(0xffffffffu, mx[q]);
+    if ((threadIdx.x & 31) == 0) atomicMax(out + q, v);
+  }
+}
+void launch_longest_rows(const CsrView &A, const CsrView &AH, int *d_out, cudaStream_t s) {
+  cudaMemsetAsync(d_out, 0, 2 * sizeof(int), s);
+  k_longest_rows<<<std::min(1024, ceil_div(A.n, 256)), 256, 0, s>>>(A, AH, d_out);
+  note_launch();
+}
+
 constexpr size_t kGatherBytes = 48u << 20;
 
 template <bool PAIR, int G>
-static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z, const cxf *P,
-                           cxf *V, int m, cudaStream_t s) {
+static void spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int longest, int ne, const cxd *d_z, int conj_z,
+                            const cxf *P, cxf *V, int m, cudaStream_t s) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -757,19 +781,42 @@ static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, c
   const size_t window = std::min<size_t>(A.n, (size_t)bw + (size_t)4 * sms * rows) * m * sizeof(cxf);
   const int ng = (int)std::min<size_t>(ne, std::max<size_t>(1, kGatherBytes / window));
   const bool few = A.nnz <= 5 * (int64_t)A.n;
-  if constexpr (PAIR && G == 32) {
-    if (few && !B && ng == ne) {
+  if constexpr (G == 32) {
+    // A warp a row against the group kernel, us, 8 nodes, 64000 rows of a stencil
+    // (50000 random ones), 48 columns, 33 where the number is odd.  Rows of five:
+    // 109 and 119, odd 115 and 109, so even numbers only.  Seven: 134 and 154 (132
+    // and 144), odd 132 and 167; complex odd the same, and beyond 48 columns slower
+    // (212 and 183).  Nine: 177 and 158, odd 173 and 171: never.  Thirteen: 232 and
+    // 314 (271 and 279), odd 249 and 390 (253 and 335).  Where nodes go in turns the
+    // row is read again in every turn, which pays from 96 columns a turn, or two
+    // passes over the row's columns (random rows of 13, a node a turn: 64 columns
+    // 804 and 656, 96 columns 513 and 591).
+    const bool turns = ng < ne && ng * m < 96 && m <= 64;
+    int K = 0;
+    if (!B && few && PAIR && ng == ne) K = 5;
+    else if (!B && !few && !turns && longest <= 7 && (PAIR || !A.cplx)) K = 7;
+    else if (!B && !turns && longest > 9 && longest <= 16 && A.nnz > 9 * (int64_t)A.n) K = 16;
+    if (K) {
+      constexpr int VW = PAIR ? 2 : 1;
       auto launch = [&](auto kern) {
         int occ = 1;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSpThreads, 0);
-        kern<<<std::min(occ * sms, need), kSpThreads, 0, s>>>(A, ne, d_z, conj_z, P, V, A.n, m);
+        kern<<<std::min(occ * sms, need), kSpThreads, 0, s>>>(A, ne, d_z, conj_z, P, V, A.n, m, ng);
+      };
+      auto pick = [&](auto cplx) {
+        constexpr bool AC = decltype(cplx)::value;
+        if constexpr (PAIR)
+          if (K == 5) return launch(k_multishift_spmm_f32_wide<AC, VW, 5>);
+        if constexpr (PAIR || !AC)
+          if (K == 7) return launch(k_multishift_spmm_f32_wide<AC, VW, 7>);
+        launch(k_multishift_spmm_f32_wide<AC, VW, 16>);
       };
       if (A.cplx)
-        launch(k_multishift_spmm_f32_wide<true>);
+        pick(std::true_type{});
       else
-        launch(k_multishift_spmm_f32_wide<false>);
+        pick(std::false_type{});
       note_launch();
-      return need;
+      return;
     }
   }
 #define SPF(AC, BC, HB, U)                                                                              \
@@ -792,19 +839,18 @@ static int spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int ne, c
   }
 #undef SPF
   note_launch();
-  return need;
 }
 
-int launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int ne, const cxd *d_z, int conj_z, const cxf *P,
-                               cxf *V, int m, cudaStream_t s) {
+void launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int longest, int ne, const cxd *d_z,
+                                int conj_z, const cxf *P, cxf *V, int m, cudaStream_t s) {
   // the fewest lanes a row that cover it in one pass
   const int cols = ceil_div(m, 2);
-#define SPG(PAIR)                                                                            \
-  do {                                                                                       \
-    if (cols <= 4) return spmm_f32_launch<PAIR, 4>(A, B, bw, ne, d_z, conj_z, P, V, m, s);   \
-    if (cols <= 8) return spmm_f32_launch<PAIR, 8>(A, B, bw, ne, d_z, conj_z, P, V, m, s);   \
-    if (cols <= 16) return spmm_f32_launch<PAIR, 16>(A, B, bw, ne, d_z, conj_z, P, V, m, s); \
-    return spmm_f32_launch<PAIR, 32>(A, B, bw, ne, d_z, conj_z, P, V, m, s);                 \
+#define SPG(PAIR)                                                                                     \
+  do {                                                                                                \
+    if (cols <= 4) return spmm_f32_launch<PAIR, 4>(A, B, bw, longest, ne, d_z, conj_z, P, V, m, s);   \
+    if (cols <= 8) return spmm_f32_launch<PAIR, 8>(A, B, bw, longest, ne, d_z, conj_z, P, V, m, s);   \
+    if (cols <= 16) return spmm_f32_launch<PAIR, 16>(A, B, bw, longest, ne, d_z, conj_z, P, V, m, s); \
+    return spmm_f32_launch<PAIR, 32>(A, B, bw, longest, ne, d_z, conj_z, P, V, m, s);                 \
   } while (0)
   if (m % 2 == 0) SPG(true);
   SPG(false);
