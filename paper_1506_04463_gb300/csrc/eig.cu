@@ -13,7 +13,11 @@
 //    balanced matrix on one CTA; Newton's method then refines all pairs at
 //    once in FP64: with R = M X - X diag(d) and E = W R, a first-order
 //    correction is X <- X (I + F), F_ij = E_ij / (d_j - d_i), d_j += E_jj, and
-//    W follows by W <- (I - F) W and Newton-Schulz steps W <- W (2 I - X W).
+//    W follows by W <- (I - F) W and Newton-Schulz steps W <- (2 I - W X) W.
+//    These are formed from the left defect I - W X because W X is what has to
+//    be the identity (Yh^H B Y = W X): in rounding the right defect differs
+//    from it by the condition number (X of condition 1e4, m = 32: |W X - I| of
+//    9e-14, of 4e-11 from the right defect, 7e-13 with an FP64 inverse).
 //    It converges quadratically where the eigenvalues are separated by more
 //    than the FP32 errors; three iterations are usual.  Where it does not get
 //    below kFTol in kMaxIt iterations (clustered or graded spectra), the FP64
@@ -558,7 +562,7 @@ __device__ __forceinline__ cxd tile_dot(const cxd *__restrict__ A, const cxd *__
 
 static dim3 tile_grid(int m, int nz = 1) { return dim3(ceil_div(m, kGn), ceil_div(m, kGm), nz); }
 
-// z = 0: R = M X - X diag(d);  z = 1: C = 2 I - X W
+// z = 0: R = M X - X diag(d);  z = 1: C = 2 I - W X
 __global__ void __launch_bounds__(128) k_eig_resid(int m, const cxd *M, const cxd *X, const cxd *W, cxd *R, cxd *C,
                                                    const EigState *st, int it) {
   __shared__ cxd sm[96];
@@ -573,11 +577,11 @@ __global__ void __launch_bounds__(128) k_eig_resid(int m, const cxd *M, const cx
       R[(size_t)i * m + j] = s;
     }
   } else {
-    const cxd s = tile_dot(X, W, m, i, j, ok, sm);
+    const cxd s = tile_dot(W, X, m, i, j, ok, sm);
     if (threadIdx.x < 32 && ok) C[(size_t)i * m + j] = mk((i == j ? 2.0 : 0.0) - s.re, -s.im);
   }
 }
-// z = 0: E = W R -> F_ij = E_ij / (d_j - d_i), d_j += E_jj;  z = 1: W1 = W C
+// z = 0: E = W R -> F_ij = E_ij / (d_j - d_i), d_j += E_jj;  z = 1: W1 = C W
 __global__ void __launch_bounds__(128) k_eig_corr(int m, const cxd *W, const cxd *R, const cxd *C, cxd *Fm, cxd *W1,
                                                   EigState *st, int it) {
   __shared__ cxd sm[96];
@@ -608,7 +612,7 @@ __global__ void __launch_bounds__(128) k_eig_corr(int m, const cxd *W, const cxd
       if (lane == 0) atomicMax(&st->fmax[it], mx);
     }
   } else {
-    const cxd s = tile_dot(W, C, m, i, j, ok, sm);
+    const cxd s = tile_dot(C, W, m, i, j, ok, sm);
     if (threadIdx.x < 32 && ok) W1[(size_t)i * m + j] = s;
   }
 }
