@@ -14,15 +14,19 @@
 // are frozen.  All phases of all refinement steps and Krylov iterations run
 // inside the one launch, separated by a grid barrier with a bounded wait.
 //
-// An iteration is six phases: v = (z I - A) y with (rh, v); alpha; s and z;
-// t = (z I - A) z with (t, s), (t, t), (rh, s), (rh, t); omega and, from
-// (rh, r) = (rh, s) - omega (rh, t), beta; then d, r, p and y in one pass over
-// the blocks.  The products read the matrix in the sweeps' precision (values
+// An iteration is eight phases, a grid barrier after each: v = (z I - A) y with
+// (rh, v); alpha; s and z; t = (z I - A) z with (t, s), (t, t); omega; d and r
+// with (r, r), (rh, r); beta and the stopping test; p and y.  ((rh, r) is summed
+// itself: from (rh, s) - omega (rh, t) the updates would be one pass over the
+// blocks and a barrier less, 1 to 10 % of an iteration on 0.3 to 3.5 million rows,
+// but FP32 sums would cancel in it.)  The products read the matrix in the sweeps' precision (values
 // converted once, at set-up: an FP64-to-FP32 conversion costs a warp 64 cycles,
 // and one for every entry, node and column was most of an iteration), a tile's
 // rows padded to one length in shared memory, two rows at a time so that some
 // eighteen gathers are in flight; the inverse diagonals come from set-up too.
-// Six problems, 13 000 rows, 8 nodes x 32 columns: 875 us an iteration before.
+// Six problems, 15 700 rows, 8 nodes x 32 columns: 895 us an iteration before,
+// 388 now; 16 problems, 336 000 rows, 8 nodes x 48 columns: 22.6 and 9.5 ms; 64
+// problems, 3.45 million rows: 208 and 85 ms.
 //
 // Layout.  Rows of all problems are concatenated; problem p owns rows
 // [off_p, off_p + n_p).  A right-hand-side / output block (Y, Q) holds
@@ -94,7 +98,7 @@ struct BatchKernelArgs {
   const cx<T> *kinv;     // 1 / (z_j - a_ii): problem p's ne x n_p at ne * off_p
   cxd *X;
   cx<T> *r, *rh, *p, *v, *y, *s, *z, *t, *d;
-  cx<T> *part;           // ntiles x 4 x PS partial dots
+  cx<T> *part;           // ntiles x 2 x PS partial dots
   double *partd;         // ntiles x PS partial |r|^2 (FP64 residual)
   double *partb;         // ntiles x m0 partial |Y_c|^2
   BatchScal sc;
@@ -110,7 +114,6 @@ struct BatchKernelArgs {
 namespace {
 
 constexpr int kEll = 2304;   // staged entries (256 rows of nine)
-constexpr int kTileMax = 256;
 
 // Rows of a tile in shared memory, padded to K entries (own row, value zero).
 template <typename T>
@@ -260,8 +263,13 @@ __device__ void for_tile_systems(const BatchKernelArgs<T> &a, TileEll<T> &e, int
 
 }  // namespace
 
-template <typename T>
-__global__ void __launch_bounds__(512) k_batch_filter(BatchKernelArgs<T> a) {
+// LEAN: FP32 in 64 registers (120 bytes of spills), for 1024 threads an SM; else
+// CTAs of at most 256 threads with up to 128 (116 used), which the short phases
+// of few rows take better.  336 000 rows in 16 problems: 9.5 ms an iteration, 12.2
+// without the lean form; a solve of six problems, 13 000 rows: 91 ms, 99 without
+// the other.  FP64 takes 128 either way and has one form.
+template <typename T, bool LEAN>
+__global__ void __launch_bounds__(LEAN ? 512 : 256, LEAN && sizeof(T) == 8 ? 1 : 2) k_batch_filter(BatchKernelArgs<T> a) {
   __shared__ TileEll<T> ell;
   const int PS = a.ne * a.m0;
   int *abort_flag = a.ctl;
@@ -375,17 +383,15 @@ __global__ void __launch_bounds__(512) k_batch_filter(BatchKernelArgs<T> a) {
             a.v[e] = o;
             cfma_cj(dot, a.rh[e], o);
           });
-          a.part[((size_t)ti * 4) * PS + j * a.m0 + c] = dot;
+          a.part[((size_t)ti * 2) * PS + j * a.m0 + c] = dot;
         });
         if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
-        // the last iteration's stopping test is complete: nobody left?
-        if (it > 0 && *(volatile int *)&a.ctl[2 + ((it - 1) & 1)] == 0) break;
         // alpha = rho / (rh, v)
         for_systems(a, [&](bool live, int s, int p, int q, int c, int sub, const BatchProb &pr) {
           const bool go = live && a.sc.act[s];
           cxd den = mk(0.0, 0.0);
           if (go)
-            for (int ti = pr.tb + sub; ti < pr.te; ti += 8) den = den + ccast<double>(a.part[((size_t)ti * 4) * PS + q]);
+            for (int ti = pr.tb + sub; ti < pr.te; ti += 8) den = den + ccast<double>(a.part[((size_t)ti * 2) * PS + q]);
           den = sum8(den);
           if (!go || sub) return;
           if (!(abs2(den) > 0) || !(den.re == den.re)) {
@@ -413,79 +419,57 @@ __global__ void __launch_bounds__(512) k_batch_filter(BatchKernelArgs<T> a) {
             zp[e] = kv * sv;
           }
         });
-        if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl[2 + (it & 1)] = 0;  // counted after this iteration's update
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl[2] = 0;  // counted after this iteration's update
         if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
-        // t = (z I - A) z ;  partial (t, s), (t, t), (rh, s), (rh, t)
+        // t = (z I - A) z ;  partial (t, s), (t, t)
         for_tile_systems<T, true, true>(a, ell, side, [&](int ti, const BatchTile &tl, const BatchProb &pr, int j, int c, int sys) {
           const int n = pr.n, m = pr.m;
           const size_t nb = (size_t)a.ne * pr.off * a.m0 + (size_t)j * n * m;
           const cx<T> zj = ccast<T>(side == 0 ? pr.z[j] : conj(pr.z[j]));
-          cx<T> ts = mk<T>(0, 0), hs = mk<T>(0, 0), ht = mk<T>(0, 0);
+          cx<T> ts = mk<T>(0, 0);
           T tt = 0;
           product(ell, pr, tl, side, zj, a.z + nb, m, c, [&](int i, cx<T> o) {
             const size_t e = nb + (size_t)i * m + c;
             a.t[e] = o;
-            const cx<T> sv = a.s[e], hv = a.rh[e];
-            cfma_cj(ts, o, sv);
-            cfma_cj(hs, hv, sv);
-            cfma_cj(ht, hv, o);
+            cfma_cj(ts, o, a.s[e]);
             tt += abs2(o);
           });
-          cx<T> *pp = a.part + ((size_t)ti * 4) * PS + j * a.m0 + c;
+          cx<T> *pp = a.part + ((size_t)ti * 2) * PS + j * a.m0 + c;
           pp[0] = ts;
           pp[PS] = mk<T>(tt, 0);
-          pp[2 * (size_t)PS] = hs;
-          pp[3 * (size_t)PS] = ht;
         });
         if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
-        // omega = (t, s) / (t, t);  rho' = (rh, s) - omega (rh, t);
-        // beta = (rho' / rho)(alpha / omega).  act = 2: breakdown, the update
-        // below is the system's last
+        // omega = (t, s) / (t, t).  act = 2: breakdown, the update below is the system's last
         for_systems(a, [&](bool live, int s, int p, int q, int c, int sub, const BatchProb &pr) {
           const bool go = live && a.sc.act[s];
-          cxd ts = mk(0.0, 0.0), hs = mk(0.0, 0.0), ht = mk(0.0, 0.0);
+          cxd ts = mk(0.0, 0.0);
           double tt = 0.0;
           if (go)
             for (int ti = pr.tb + sub; ti < pr.te; ti += 8) {
-              const cx<T> *pp = a.part + ((size_t)ti * 4) * PS + q;
+              const cx<T> *pp = a.part + ((size_t)ti * 2) * PS + q;
               ts = ts + ccast<double>(pp[0]);
               tt += (double)pp[PS].re;
-              hs = hs + ccast<double>(pp[2 * (size_t)PS]);
-              ht = ht + ccast<double>(pp[3 * (size_t)PS]);
             }
           ts = sum8(ts);
           tt = sum8(tt);
-          hs = sum8(hs);
-          ht = sum8(ht);
           if (!go || sub) return;
           const cxd om = tt > 0 ? (1.0 / tt) * ts : mk(0.0, 0.0);
           a.sc.omega[s] = om;
-          if (!(abs2(om) > 0) || !(abs2(a.sc.rho[s]) > 0)) {
-            a.sc.beta[s] = mk(0.0, 0.0);
-            a.sc.act[s] = 2;
-            return;
-          }
-          cxd hr = hs;
-          cfms(hr, om, ht);
-          a.sc.beta[s] = cdiv(hr, a.sc.rho[s]) * cdiv(a.sc.alpha[s], om);
-          a.sc.rho[s] = hr;
+          if (!(abs2(om) > 0) || !(abs2(a.sc.rho[s]) > 0)) a.sc.act[s] = 2;
         });
         if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
-        // d += alpha y + omega z ; r = s - omega t ; p = r + beta (p - omega v) ;
-        // y = K^{-1} p ; partial (r, r)
+        // d += alpha y + omega z ; r = s - omega t ; partial (r, r), (rh, r)
         for_tile_systems<T, true, false>(a, ell, side, [&](int ti, const BatchTile &tl, const BatchProb &pr, int j, int c, int sys) {
           const int n = pr.n, m = pr.m;
           const size_t nb = (size_t)a.ne * pr.off * a.m0 + (size_t)j * n * m;
           const cx<T> al = ccast<T>(a.sc.alpha[sys]);
           const cx<T> om = ccast<T>(a.sc.omega[sys]);
-          const cx<T> be = ccast<T>(a.sc.beta[sys]);
-          const cx<T> *ki = a.kinv + (size_t)a.ne * pr.off + (size_t)j * n;
           const cx<T> *__restrict__ zp = a.z + nb + c, *__restrict__ sp = a.s + nb + c, *__restrict__ tp = a.t + nb + c,
-                      *__restrict__ vp = a.v + nb + c;
-          cx<T> *__restrict__ dp = a.d + nb + c, *__restrict__ yp = a.y + nb + c, *__restrict__ rp = a.r + nb + c,
-                *__restrict__ pp = a.p + nb + c;
+                      *__restrict__ yp = a.y + nb + c, *__restrict__ hp = a.rh + nb + c;
+          cx<T> *__restrict__ dp = a.d + nb + c, *__restrict__ rp = a.r + nb + c;
           T rr2 = 0;
-#pragma unroll 2
+          cx<T> hr = mk<T>(0, 0);
+#pragma unroll 4
           for (int i = tl.r0; i < tl.r1; ++i) {
             const size_t e = (size_t)i * m;
             cx<T> dv = dp[e];
@@ -496,34 +480,62 @@ __global__ void __launch_bounds__(512) k_batch_filter(BatchKernelArgs<T> a) {
             cfms(rv, om, tp[e]);
             rp[e] = rv;
             rr2 += abs2(rv);
+            cfma_cj(hr, hp[e], rv);
+          }
+          cx<T> *pp = a.part + ((size_t)ti * 2) * PS + j * a.m0 + c;
+          pp[0] = hr;
+          pp[PS] = mk<T>(rr2, 0);
+        });
+        if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
+        // stop on |r|^2 <= stop2 or breakdown; beta = ((rh, r) / rho)(alpha / omega) of the others
+        for_systems(a, [&](bool live, int s, int p, int q, int c, int sub, const BatchProb &pr) {
+          const int act = live ? a.sc.act[s] : 0;
+          double rr2 = 0.0;
+          cxd hr = mk(0.0, 0.0);
+          if (act)
+            for (int ti = pr.tb + sub; ti < pr.te; ti += 8) {
+              const cx<T> *pp = a.part + ((size_t)ti * 2) * PS + q;
+              hr = hr + ccast<double>(pp[0]);
+              rr2 += (double)pp[PS].re;
+            }
+          rr2 = sum8(rr2);
+          hr = sum8(hr);
+          __syncwarp();
+          if (!act || sub) return;
+          if (act == 2 || !(rr2 > a.sc.stop2[s]) || !(rr2 == rr2)) {
+            a.sc.act[s] = 0;
+            return;
+          }
+          a.sc.beta[s] = cdiv(hr, a.sc.rho[s]) * cdiv(a.sc.alpha[s], a.sc.omega[s]);
+          a.sc.rho[s] = hr;
+          atomicAdd(&a.ctl[2], 1);
+        });
+        if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
+        if (*(volatile int *)&a.ctl[2] == 0) {  // nobody left
+          ++it;
+          break;
+        }
+        // p = r + beta (p - omega v) ;  y = K^{-1} p
+        for_tile_systems<T, true, false>(a, ell, side, [&](int ti, const BatchTile &tl, const BatchProb &pr, int j, int c, int sys) {
+          const int n = pr.n, m = pr.m;
+          const size_t nb = (size_t)a.ne * pr.off * a.m0 + (size_t)j * n * m;
+          const cx<T> om = ccast<T>(a.sc.omega[sys]);
+          const cx<T> be = ccast<T>(a.sc.beta[sys]);
+          const cx<T> *ki = a.kinv + (size_t)a.ne * pr.off + (size_t)j * n;
+          const cx<T> *__restrict__ vp = a.v + nb + c, *__restrict__ rp = a.r + nb + c;
+          cx<T> *__restrict__ yp = a.y + nb + c, *__restrict__ pp = a.p + nb + c;
+#pragma unroll 4
+          for (int i = tl.r0; i < tl.r1; ++i) {
+            const size_t e = (size_t)i * m;
             cx<T> tmp = pp[e];
             cfms(tmp, om, vp[e]);
-            cx<T> pv = rv;
+            cx<T> pv = rp[e];
             cfma(pv, be, tmp);
             pp[e] = pv;
             const cx<T> kv = side == 0 ? ki[i] : conj(ki[i]);
             yp[e] = kv * pv;
           }
-          a.part[((size_t)ti * 4) * PS + j * a.m0 + c] = mk<T>(rr2, 0);
         });
-        if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
-        // stop on |r|^2 <= stop2 or breakdown; the count is read after the next
-        // product's barrier (a system that stops may still be multiplied once:
-        // its v is not used)
-        for_systems(a, [&](bool live, int s, int p, int q, int c, int sub, const BatchProb &pr) {
-          const int act = live ? a.sc.act[s] : 0;
-          double rr2 = 0.0;
-          if (act)
-            for (int ti = pr.tb + sub; ti < pr.te; ti += 8) rr2 += (double)a.part[((size_t)ti * 4) * PS + q].re;
-          rr2 = sum8(rr2);
-          __syncwarp();
-          if (!act || sub) return;
-          if (act == 2 || !(rr2 > a.sc.stop2[s]) || !(rr2 == rr2))
-            a.sc.act[s] = 0;
-          else
-            atomicAdd(&a.ctl[2 + (it & 1)], 1);
-        });
-        // the partial sums read above are written again by the next product
         if (!grid_bar(a.bar, abort_flag, a.err, a.spin_limit)) return;
       }
       kry_total += it;
@@ -620,14 +632,20 @@ static BatchKernelArgs<T> make_args(const BatchLaunch &L) {
 }
 
 template <typename T>
-int batch_filter_max_ctas_per_sm(int threads) {
+static const void *batch_kernel(bool lean) {
+  if constexpr (sizeof(T) == 4)
+    if (!lean) return (const void *)k_batch_filter<T, false>;
+  return (const void *)k_batch_filter<T, true>;
+}
+template <typename T>
+int batch_filter_max_ctas_per_sm(int threads, bool lean) {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_filter<T>, threads, 0) != cudaSuccess) nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel<T>(lean), threads, 0) != cudaSuccess) nb = 0;
   cudaGetLastError();
   return nb;
 }
-template int batch_filter_max_ctas_per_sm<float>(int);
-template int batch_filter_max_ctas_per_sm<double>(int);
+template int batch_filter_max_ctas_per_sm<float>(int, bool);
+template int batch_filter_max_ctas_per_sm<double>(int, bool);
 
 template <typename T>
 cudaError_t batch_filter_launch(const BatchLaunch &L, int grid, int threads, cudaStream_t s) {
@@ -639,7 +657,7 @@ cudaError_t batch_filter_launch(const BatchLaunch &L, int grid, int threads, cud
   if (e != cudaSuccess) return e;
   BatchKernelArgs<T> a = make_args<T>(L);
   void *params[] = {&a};
-  e = cudaLaunchCooperativeKernel((const void *)k_batch_filter<T>, dim3(grid), dim3(threads), params, 0, s);
+  e = cudaLaunchCooperativeKernel(batch_kernel<T>(L.lean), dim3(grid), dim3(threads), params, 0, s);
   note_launch();
   return e;
 }

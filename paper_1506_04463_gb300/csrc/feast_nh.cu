@@ -1806,32 +1806,41 @@ void batch_autotune(feast_nh_batch *b) {
   launch_fill_pattern(b->Yh, b->ntot * b->m0, b->s);
   float best = 1e30f;
   int bt = 256, bg = 0, br = 128;
-  const int threads_c[] = {256, 512};
+  bool bl = false;
+  const struct {
+    int threads, per_sm;
+    bool lean;
+  } shapes[] = {{256, 1, false}, {256, 2, false}, {256, 4, true}, {512, 1, true}, {512, 2, true}};
+  // 256 rows never won: 8 nodes, 48 columns, ms an iteration with 16, 64 and 256
+  // rows a tile 8.5, 8.6 and 13.3 at 336 000 rows in 16 problems, 79.7, 83.6 and
+  // 115 at 3.45 million in 64
   const int rows_c[] = {16, 64};
   b->L.side1 = 0;  // one side is enough to compare shapes
   BCK(cudaEventRecord(b->ev[2], b->s));
-  for (int th : threads_c) {
-    const int occ = batch_fp32(b) ? batch_filter_max_ctas_per_sm<float>(th) : batch_filter_max_ctas_per_sm<double>(th);
-    if (occ < 1) continue;
-    for (int per_sm = 1; per_sm <= std::min(occ, 4); per_sm *= 2)
-      for (int rows : rows_c) {
-        batch_tiles(b, rows);
-        b->threads = th;
-        b->grid = std::min(sms * per_sm, std::max(1, b->ntiles));
-        batch_filter_run(b, 0.0, 1, 3);
-        BCK(cudaEventRecord(b->ev[0], b->s));
-        batch_filter_run(b, 0.0, 1, 3);
-        BCK(cudaEventRecord(b->ev[1], b->s));
-        BCK(cudaEventSynchronize(b->ev[1]));
-        float ms = 0;
-        BCK(cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]));
-        if (ms < best) {
-          best = ms;
-          bt = th;
-          bg = b->grid;
-          br = rows;
-        }
+  for (const auto &sh : shapes) {
+    const int occ = batch_fp32(b) ? batch_filter_max_ctas_per_sm<float>(sh.threads, sh.lean)
+                                  : batch_filter_max_ctas_per_sm<double>(sh.threads, sh.lean);
+    if (occ < sh.per_sm) continue;
+    for (int rows : rows_c) {
+      batch_tiles(b, rows);
+      b->threads = sh.threads;
+      b->L.lean = sh.lean;
+      b->grid = std::min(sms * sh.per_sm, std::max(1, b->ntiles));
+      batch_filter_run(b, 0.0, 1, 3);
+      BCK(cudaEventRecord(b->ev[0], b->s));
+      batch_filter_run(b, 0.0, 1, 3);
+      BCK(cudaEventRecord(b->ev[1], b->s));
+      BCK(cudaEventSynchronize(b->ev[1]));
+      float ms = 0;
+      BCK(cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]));
+      if (ms < best) {
+        best = ms;
+        bt = sh.threads;
+        bg = b->grid;
+        br = rows;
+        bl = sh.lean;
       }
+    }
   }
   b->L.side1 = 1;
   BCK(cudaEventRecord(b->ev[3], b->s));
@@ -1842,6 +1851,7 @@ void batch_autotune(feast_nh_batch *b) {
   BREQ(bg > 0, "no launch shape of the batched solver fits this device");
   b->threads = bt;
   b->grid = bg;
+  b->L.lean = bl;
   batch_tiles(b, br);
   int herr = 0;
   BCK(cudaMemcpyAsync(&herr, b->L.err, sizeof(int), cudaMemcpyDeviceToHost, b->s));
@@ -1973,7 +1983,7 @@ feast_nh_status feast_nh_batch_init(feast_nh_batch **out, int32_t nprob, const f
     b->dtiles = balloc<BatchTile>(b, (size_t)maxt * sizeof(BatchTile));
     b->dprob = balloc<BatchProb>(b, (size_t)nprob * sizeof(BatchProb));
     const size_t PS = (size_t)ne * m0;
-    b->L.part = balloc<void>(b, (size_t)maxt * 4 * PS * es);
+    b->L.part = balloc<void>(b, (size_t)maxt * 2 * PS * es);
     b->L.partd = balloc<double>(b, (size_t)maxt * PS * sizeof(double));
     b->L.partb = balloc<double>(b, (size_t)maxt * m0 * sizeof(double));
     const size_t S = (size_t)nprob * PS;

@@ -168,6 +168,7 @@ struct BatchLaunch {
   const cxd *Y, *Yh;
   cxd *Q, *Qh;
   const void *kinv; // 1 / (z_j - a_ii), ne x n per problem
+  bool lean;        // which form of the kernel
   cxd *X;
   void *kblk[9];   // r, rh, p, v, y, s, z, t, d in the Krylov precision
   void *part;
@@ -185,7 +186,9 @@ struct BatchLaunch {
 // (float: FP32 Krylov sweeps + FP64 refinement; double: plain FP64).
 template <typename T>
 cudaError_t batch_filter_launch(const BatchLaunch &L, int grid, int threads, cudaStream_t s);
-template <typename T> int batch_filter_max_ctas_per_sm(int threads);
+// lean: fewer registers (FP32), so that more threads are resident; up to 512
+// threads a CTA, else up to 256.
+template <typename T> int batch_filter_max_ctas_per_sm(int threads, bool lean);
 // Values and inverse diagonals of one problem in the sweeps' precision.
 template <typename T>
 void launch_batch_setup(const CsrView &A, const CsrView &AH, const cxd *diag, const cxd *z, int ne, T *vA, T *vAH,
