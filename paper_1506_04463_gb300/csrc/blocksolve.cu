@@ -188,8 +188,9 @@ __device__ __forceinline__ void put(cxf *t, int b, int line, int x, cxf v) {
 
 // ---------------------------------------------------------------------------
 // off-diagonal entries: row r's entries of M = z B - A in the block before
-// (dir 0) and after (dir 1) its own, K a row (local column, -1 terminated by
-// zero values at column 0), values of A and of B apart since z differs by node
+// (dir 0) and after (dir 1) its own, K a row (local column; rows with fewer are
+// filled up with zeros at column 0), values of A and of B apart since z differs
+// by node
 // ---------------------------------------------------------------------------
 __global__ void k_block_count(CsrView A, CsrView B, int hasB, int b, int *kmax) {
   int mx = 0;
@@ -249,8 +250,8 @@ __global__ void k_block_entries(CsrView A, CsrView B, int hasB, int b, int K, in
 // and backward substitution on 16-row blocks, whose diagonal inverses are
 // there already (k_band_diag_inv).  Y (b x 32) stays in shared memory; a
 // 16-row strip of the factor is staged for each block; four rows a warp, the
-// sum over k in two halves.  FP arithmetic of the factors' precision, 18 M
-// complex FMAs a block at b = 304, all blocks of all factors independent.
+// sum over k in two halves.  FP arithmetic of the factors' precision, 2/3 b^3
+// complex FMAs a block (11 M at b = 256), all blocks of all factors independent.
 // Output: column-major (Tc, for M) and row-major (Tr, for M^H) copies.
 // ---------------------------------------------------------------------------
 template <typename T>

@@ -830,10 +830,10 @@ int do_rr(feast_nh_ctx *ctx, const cxd *Q, const cxd *Qh, int m, cxd *Y, cxd *Yh
     BQq = ctx->T1;
   }
   proj_gram(ctx, Qh, m, m, BQq, m, m, ctx->BQ);
-  // 3.a-3.c: coefficients of U, Uh with Uh^H B U = I, 2.b spurious.  Usually
-  // by elimination (no column can be dropped); otherwise, and for the bilinear
-  // form of a complex symmetric pencil, by B_Q = V Gamma V^^H with the resize
-  // and sort of eq. (resize).
+  // 3.a-3.c: coefficients of U, Uh with Uh^H B U = I, 2.b spurious.  By
+  // elimination where provably no column can be dropped (B_Q is not graded);
+  // otherwise, and for the bilinear form of a complex symmetric pencil, by B_Q =
+  // V Gamma V^^H with the resize and sort of eq. (resize).
   bool eig = cs;
   if (!cs) {
     CKC(launch_biorth(m, ctx->BQ, ctx->prev_rho, ctx->prev_inside, ctx->have_prev, ctx->o.mu, ctx->o.eta, ctx->S,

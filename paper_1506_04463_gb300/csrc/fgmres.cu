@@ -8,9 +8,9 @@
 // and Givens rotations; the block kernels below run all systems in one pass:
 // node-major blocks ne x n x m (row-major n x m per node, complex float),
 // system s = j*m + c.  Orthogonalisation is classical Gram-Schmidt applied
-// twice (one pass for the dot products of all previous basis vectors, one
-// for the update, repeated).  Scalars and the small least-squares problems
-// are FP64.  Converged systems are frozen (their columns are skipped).
+// twice, in three passes over the block: dot products with all previous basis
+// vectors; update and dot products again; update and norm.  Scalars and the
+// small least-squares problems are FP64.  Converged systems are frozen (their columns are skipped).
 #include <algorithm>
 #include <vector>
 
