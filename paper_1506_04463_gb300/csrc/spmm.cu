@@ -689,7 +689,10 @@ template <int VW> __device__ __forceinline__ void storew(cxf *p, float4 v) {
 // nodes at a time.  Bound by the gathers out of L2, K + 1 in flight
 // a lane; the group kernel above spends as many issue slots on its shuffles,
 // and past nine entries it has no row in registers.  What each K measured
-// against it stands with the rule below.
+// against it stands with the rule below.  Real rows of five (all nodes at once)
+// take complex products and the column in each row's address, which the compiler
+// schedules better there: 300 x 300 grid, 64 columns, 16 nodes 298 us, 302 in the
+// other form; complex ones 253 and 234.
 template <bool ACPLX, int VW, int K>
 __global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView A, int ne, const cxd *__restrict__ z,
                                                                          int conj_z, const cxf *__restrict__ P,
@@ -711,8 +714,9 @@ __global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView
     }
     return mk(-(float)A.val[k], 0.f);
   };
-  for (int j0 = 0; j0 < ne; j0 += ng) {
-    const int j1 = min(ne, j0 + ng);
+  constexpr bool FIVE = K == 5 && !ACPLX;
+  for (int j0 = 0; j0 < ne; j0 += FIVE ? ne : ng) {
+    const int j1 = FIVE ? ne : min(ne, j0 + ng);
     for (int i = warp; i < n; i += nwarps) {
       const int64_t ka = A.rowptr[i];
       const int nk = (int)(A.rowptr[i + 1] - ka);
@@ -727,19 +731,20 @@ __global__ void __launch_bounds__(kSpThreads) k_multishift_spmm_f32_wide(CsrView
       for (int c = lane * VW; c < m; c += 32 * VW) {
 #pragma unroll 2
         for (int j = j0; j < j1; ++j) {
-          const cxf *Pj = P + (size_t)j * xns + c;
+          const cxf *Pj = P + (size_t)j * xns + (FIVE ? 0 : c);
+          const int cj = FIVE ? c : 0;
           float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
           if (fast) {
             float4 xs[K];
 #pragma unroll
-            for (int k = 0; k < K; ++k) xs[k] = loadw<VW>(Pj + (size_t)col[k] * m);
-            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m));
+            for (int k = 0; k < K; ++k) xs[k] = loadw<VW>(Pj + (size_t)col[k] * m + cj);
+            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m + cj));
 #pragma unroll
-            for (int k = 0; k < K; ++k) vfma<ACPLX>(acc, av[k], xs[k]);
+            for (int k = 0; k < K; ++k) vfma<ACPLX || FIVE>(acc, av[k], xs[k]);
           } else {
-            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m));
+            vfma<true>(acc, zs[j], loadw<VW>(Pj + (size_t)i * m + cj));
             for (int k = 0; k < nk; ++k)
-              vfma<ACPLX>(acc, entry(ka + k), loadw<VW>(Pj + (size_t)A.colind[ka + k] * m));
+              vfma<ACPLX || FIVE>(acc, entry(ka + k), loadw<VW>(Pj + (size_t)A.colind[ka + k] * m + cj));
           }
           storew<VW>(V + (size_t)j * xns + (size_t)i * m + c, acc);
         }
