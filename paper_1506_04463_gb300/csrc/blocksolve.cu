@@ -348,8 +348,12 @@ struct BlockArgs {
 // grid (column groups, nodes, sides).  Two groups of 256 consumer threads and
 // one producer warp, which streams the tiles of T, eight columns at a time,
 // through shared memory with bulk copies (full / empty mbarriers, bounded
-// waits).  The groups take alternate stages and their sums are added through
-// shared memory.  (One group, two warps a sub-partition, left the FMA pipe idle
+// waits).  The groups take alternate chunks, each with full mbarriers of its own,
+// and their sums are added through shared memory.  (With an odd number of stages
+// both groups meet every stage, in turns.  On full barriers shared by the groups
+// each would see every second phase only, and a wait by parity for phase p + 2
+// passes while p + 1 is still being filled: copies may land out of order, and a
+// warp without rows gets there first.)  (One group, two warps a sub-partition, left the FMA pipe idle
 // half of the time; copies issued by a consumer thread delayed its warp and
 // with it everyone.)
 // A step: the right-hand side of the product, t = source - M_{i,i-1} z
@@ -381,18 +385,20 @@ __global__ void __launch_bounds__(kCons + 32, 1)
   cx<T> *va = src + (size_t)b * R;                                   // b x K entries of A
   cx<T> *vb = va + (size_t)b * K;                                    // ... of B (if any)
   int *ix = reinterpret_cast<int *>(vb + (io.vb[0] ? (size_t)b * K : 0));  // b x K local columns
-  uint64_t *full = reinterpret_cast<uint64_t *>(ix + (size_t)b * K);
-  uint64_t *empty = full + kMaxStages;
+  uint64_t *full = reinterpret_cast<uint64_t *>(ix + (size_t)b * K);  // of group g and stage s at g kMaxStages + s
+  uint64_t *empty = full + 2 * kMaxStages;
+  const int period = (stages & 1) ? stages : stages / 2;  // chunks of a group between two uses of a stage
   const int tid = threadIdx.x;
   if (tid == 0) {
     for (int s = 0; s < stages; ++s) {
       mbar::init(&full[s], 1);
+      mbar::init(&full[kMaxStages + s], 1);
       mbar::init(&empty[s], kGroup / 32);
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();
-  const int nch = b / KC;                         // stages of one product
+  const int nch = b / KC;                         // chunks of one product (even)
   const int nsteps = 2 * nblk - 1;
   const cx<T> *Tb = (side ? Tr : Tc) + (size_t)slot * nblk * b * b;
   auto block_of = [&](int s) { return s < nblk ? s : 2 * nblk - 2 - s; };
@@ -410,8 +416,9 @@ __global__ void __launch_bounds__(kCons + 32, 1)
             ok = false;
             break;
           }
-          mbar::expect_tx(&full[s], bytes);
-          mbar::bulk_load(stage + (size_t)s * tile, g, bytes, &full[s]);
+          uint64_t *f = &full[(c & 1) * kMaxStages + s];
+          mbar::expect_tx(f, bytes);
+          mbar::bulk_load(stage + (size_t)s * tile, g, bytes, f);
           ++pending;
           if (++s == stages) {
             s = 0;
@@ -422,7 +429,8 @@ __global__ void __launch_bounds__(kCons + 32, 1)
       if (!ok) {
         atomicOr(err, DEVERR_TIMEOUT);
         // copies still in flight land (bounded) before the shared memory is given up
-        for (int k = max(0, pending - stages); k < pending; ++k) mbar::wait(&full[k % stages], (k / stages) & 1, kSpin);
+        for (int k = max(0, pending - stages); k < pending; ++k)
+          mbar::wait(&full[(k & 1) * kMaxStages + k % stages], (k / 2 / period) & 1, kSpin);
       }
     }
     return;
@@ -441,9 +449,14 @@ __global__ void __launch_bounds__(kCons + 32, 1)
   const cx<T> zn = mk<T>((T)zz.re, side ? (T)-zz.im : (T)zz.im);
   const size_t dirs = (size_t)nblk * b * K;
   bool dead = false;
-  int st = half % stages, par = (half / stages) & 1;  // stage of the group's next chunk, and its parity
-  auto advance = [&](int d) {
-    for (st += d; st >= stages; st -= stages) par ^= 1;
+  int st = half, uses = 0, par = 0;  // the group's next chunk: its stage, and the parity of that stage's use
+  auto advance = [&]() {
+    st += 2;
+    if (st >= stages) st -= stages;
+    if (++uses == period) {
+      uses = 0;
+      par ^= 1;
+    }
   };
   Prod prod;
 
@@ -500,14 +513,14 @@ __global__ void __launch_bounds__(kCons + 32, 1)
     // ---- product ----
     prod.zero();
     for (int ch = half; ch < nch; ch += 2) {
-      if (!dead && !mbar::wait(&full[st], par, kSpin)) {
+      if (!dead && !mbar::wait(&full[half * kMaxStages + st], par, kSpin)) {
         dead = true;
         atomicOr(err, DEVERR_TIMEOUT);
       }
       if (act && !dead) prod.stage(stage + (size_t)st * tile, tb + (size_t)ch * KC * R + cg * C, b, R, rg, RG);
       __syncwarp();
       if ((tid & 31) == 0) mbar::arrive(&empty[st]);
-      advance(2);
+      advance();
     }
     // zb is not read any more in this step: the second group's sums, then the
     // solution of the block
@@ -559,7 +572,7 @@ static int sm_count() {
 template <typename T> static size_t solve_bytes(int b, int R, int K, bool hasB, int stages) {
   const size_t es = sizeof(cx<T>), rs = sizeof(typename Product<T, 1, 1>::Rhs);
   return ((size_t)stages * Chunk<T>::KC * b + 2 * (size_t)b * R + (size_t)(hasB ? 2 : 1) * b * K) * es +
-         (size_t)b * R * rs + (size_t)b * K * sizeof(int) + 2 * kMaxStages * sizeof(uint64_t);
+         (size_t)b * R * rs + (size_t)b * K * sizeof(int) + 3 * kMaxStages * sizeof(uint64_t);
 }
 template <typename T> static size_t inv_bytes(int b) {
   return ((size_t)b * 33 + 16 * (size_t)(b + 2) + 2 * 512 + 16 * 17) * sizeof(cx<T>);

@@ -141,3 +141,23 @@ def test_no_room_for_the_inverses():
         free()
     for a, b, y in zip(out, ref, Y):
         assert np.all(np.linalg.norm(a - b, axis=0) <= 2 * (TOL + 1e-13) * np.linalg.norm(host(y), axis=0))
+
+
+@pytest.mark.parametrize("prec,n,bw,m,ne,far", [
+    (F.PREC_FP64, 8000, 208, 8, 4, 1), (F.PREC_FP64, 8000, 224, 8, 4, 1), (F.PREC_FP64, 8000, 112, 16, 8, 1),
+    (F.PREC_FP64, 4000, 48, 32, 8, 1), (F.PREC_FP32_IR, 5000, 240, 64, 8, 8)])
+def test_odd_number_of_stages(prec, n, bw, m, ne, far):
+    """Three stages (FP64) and five (FP32, blocks of 240 with eight entries towards a neighbour), which the two groups
+    of a product use in turns, some warps without rows of their own: bit-identical results, filter after filter, by a
+    solve that needs no other form."""
+    rng = np.random.default_rng(bw)
+    offs = [o for k in range(far) for o in (bw - k, k - bw)] + ([1, -7] if far < 7 else [])  # at most eight either way
+    A = (sp.diags([rng.uniform(-1, 1, n - abs(o)) for o in offs], offs) + (6 + len(offs)) * sp.eye(n)).tocsr()
+    con = wl.Contour(0, 4 + 0.1j, 1.0, ne=ne)
+    Y = [dev(rng.standard_normal((n, m))) for _ in range(2)]
+    ctx = F.FeastNH(A, None, con, m, precision=prec, inner_tol=TOL)
+    ref = [q.clone() for q in ctx.filter(*Y)]
+    for _ in range(6):
+        assert all(torch.equal(a, b) for a, b in zip(ctx.filter(*Y), ref))
+    assert ctx.forms() & F.FORM_BLOCKS
+    ctx.close()
