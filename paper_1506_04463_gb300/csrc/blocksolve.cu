@@ -608,6 +608,17 @@ int block_size(int kl, int ku) { return std::max(16, ceil_div(std::max(kl, ku), 
 // n = 90000) and the inverses 35 ms, and more refinement steps are needed.
 constexpr int kMaxBlock = 256;
 bool block_solve_fits(int kl, int ku) { return block_size(kl, ku) <= kMaxBlock; }
+// FP64: a filter takes two sweeps (the refinement), each bound by the FP64 pipe,
+// so that its time goes with the number of rounds that its CTAs of four columns
+// make on the chip; the triangular solves are one chain of windows whatever the
+// columns.  8000 rows, ms a filter in 1, 2, 3, 4 rounds against the factors: b =
+// 16 5.7, 11.6, 17.2, 22.9 and 20; b = 48 7.5, 15, 23, 30 and 28; b = 112 15, 30,
+// 45, 60 and 45; b = 176 25, 50, 75, 100 and 66 to 72; b = 256 33, 66, 99, 132 and
+// 88 to 94.
+bool block_solve_pays_f64(int kl, int ku, int m, int ne, int nsides) {
+  const int rounds = ceil_div(ceil_div(m, kGroups) * ne * nsides, sm_count());
+  return rounds <= (block_size(kl, ku) <= 96 ? 3 : 2);
+}
 
 // Largest number of off-diagonal entries of a row towards one block into
 // *d_kmax (zeroed by the caller).

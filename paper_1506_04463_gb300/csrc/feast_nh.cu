@@ -1124,7 +1124,8 @@ void init_ctx(feast_nh_ctx *ctx, const feast_nh_csr *A, const feast_nh_csr *B, c
       // the triangular factors, so that opts have to allow one
       const bool room = f32 || ctx->o.inner_max > 1;
       ctx->tri = room && ctx->kl <= 1 && ctx->ku <= 1;
-      if (room && !ctx->tri && block_solve_fits(ctx->kl, ctx->ku)) {
+      if (room && !ctx->tri && block_solve_fits(ctx->kl, ctx->ku) &&
+          (f32 || block_solve_pays_f64(ctx->kl, ctx->ku, m0, ne, cs_mode(ctx) ? 1 : 2))) {
         // off-diagonal entries of a row between blocks, both sides
         int *d_k = dalloc<int>(ctx, sizeof(int)), hk = 0;
         CKC(cudaMemsetAsync(d_k, 0, sizeof(int), ctx->s));

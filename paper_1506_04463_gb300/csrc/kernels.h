@@ -55,6 +55,7 @@ struct BlockEntries {
 int block_size(int kl, int ku);
 constexpr int kBlockMaxEntries = 8;  // off-diagonal entries of a row towards a neighbouring block at most
 bool block_solve_fits(int kl, int ku);
+bool block_solve_pays_f64(int kl, int ku, int m, int ne, int nsides);  // against the triangular solves
 void launch_block_count(const CsrView &A, const CsrView *B, int kl, int ku, int *d_kmax, cudaStream_t s);
 size_t block_entry_count(int n, int kl, int ku, int K);
 template <typename T>

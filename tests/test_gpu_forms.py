@@ -13,7 +13,7 @@ import scipy.sparse as sp  # noqa: E402
 
 from paper_1506_04463_gb300 import feast_nh as F  # noqa: E402
 from paper_1506_04463_gb300 import workloads as wl  # noqa: E402
-from gpu_helpers import dev, make_ctx  # noqa: E402
+from gpu_helpers import dev, host, make_ctx  # noqa: E402
 import test_gpu_small_eig  # noqa: E402
 from test_gpu_solve_forms import TOL, _band, _run  # noqa: E402
 
@@ -88,3 +88,27 @@ def test_rayleigh_ritz(made, monkeypatch, m):
     test_gpu_small_eig.test_rayleigh_ritz_sizes(m)
     small = F.FORM_ELIMINATION | F.FORM_NEAR_IDENTITY | (F.FORM_EIG_REFINED if m >= 4 else 0)
     assert made[0].forms() & ~SOLVES == small
+
+
+@pytest.mark.parametrize("bw,m,ne,blocks", [(4, 64, 14, True), (4, 64, 15, False), (90, 24, 25, True), (96, 32, 28, True),
+                                            (97, 32, 19, True), (97, 32, 20, False), (256, 128, 16, False)])
+def test_fp64_blocks_by_rounds(bw, m, ne, blocks):
+    """The FP64 rule at its line on a chip of 152 SMs: CTAs of four columns, two sides, three rounds for blocks of up to
+    96 rows and two for larger ones; the filter is right either way."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the line depends on the number of SMs")
+    n = 700
+    A = _band(n, bw, bw, bw, False)
+    con = wl.Contour(0, 4 + 0.1j, 1.0, ne=ne)
+    ctx = F.FeastNH(A, None, con, m, precision=F.PREC_FP64, inner_tol=TOL)
+    Y = np.random.default_rng(1).standard_normal((n, m))
+    Q, _ = ctx.filter(dev(Y), dev(Y))
+    assert (ctx.forms() & SOLVES == F.FORM_BLOCKS) == blocks
+    ctx.close()
+    z, w = F.nodes(con)
+    ref, amp = 0, 0.0
+    for zj, wj in zip(z, w):
+        inv = np.linalg.inv(zj * np.eye(n) - A.toarray())
+        ref, amp = ref + wj * (inv @ Y), amp + abs(wj) * np.linalg.norm(inv, 2)
+    err = np.linalg.norm(host(Q) - ref, axis=0)
+    assert np.all(err <= (TOL + 1e-13) * amp * np.linalg.norm(Y, axis=0))
