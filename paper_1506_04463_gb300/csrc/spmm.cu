@@ -45,7 +45,10 @@ constexpr int kMsMaxPairs = 8;  // ne*m <= 2048
 constexpr int kMsRows = 8;      // rows between two barriers
 constexpr int kMsStage = 160;   // entries of A they may have to be staged
 
-template <typename Tout, bool ACPLX, bool BCPLX, bool HASB>
+// LONG: rows of more than 128 entries on average, nothing staged or folded, since
+// the search for the diagonal takes more than it saves there (600 full rows, 8
+// nodes, 1, 13 and 32 columns 170, 226 and 384 us folded, 142, 175 and 335 so).
+template <typename Tout, bool ACPLX, bool BCPLX, bool HASB, bool LONG = false>
 __global__ void __launch_bounds__(kMsThreads, 4)
     k_multishift_residual(CsrView A, CsrView B, int ne, const cxd *__restrict__ z,
                           const cxd *__restrict__ w, const cxd *__restrict__ X, size_t xns,
@@ -53,13 +56,14 @@ __global__ void __launch_bounds__(kMsThreads, 4)
                           double *__restrict__ partial, int m, int rows_per_cta, const int *skip) {
   if (skip && *skip) return;
   using Val = typename std::conditional<ACPLX, cxd, double>::type;
-  __shared__ cxd ws[kMaxNe], zs[HASB ? 1 : kMsRows][kMaxNe];
+  constexpr bool FOLD = !HASB && !LONG;
+  __shared__ cxd ws[kMaxNe], zs[FOLD ? kMsRows : 1][kMaxNe];
   __shared__ Val sval[kMsStage];
   __shared__ int scol[kMsStage], sbeg[kMsRows], send[kMsRows];
   const int tid = threadIdx.x;
   if (tid < ne) {
     ws[tid] = w[tid];
-    if (HASB) zs[0][tid] = z[tid];
+    if (!FOLD) zs[0][tid] = z[tid];
   }
   const int P = ne * m;
   const int n = A.n;
@@ -72,9 +76,9 @@ __global__ void __launch_bounds__(kMsThreads, 4)
   for (int i0 = rbeg; i0 < rend; i0 += kMsRows) {
     const int rows = min(kMsRows, rend - i0);
     const int64_t k0 = A.rowptr[i0];
-    const bool staged = A.rowptr[i0 + rows] - k0 <= kMsStage;
+    const bool staged = !LONG && A.rowptr[i0 + rows] - k0 <= kMsStage;
     __syncthreads();
-    if (!HASB) {
+    if (FOLD) {
       // z_j - a_ii of the chunk's rows (entries of one position add up)
       for (int e = tid; e < rows * ne; e += kMsThreads) {
         const int r = e / ne, j = e - r * ne, i = i0 + r;
@@ -90,7 +94,7 @@ __global__ void __launch_bounds__(kMsThreads, 4)
       sbeg[r] = o;
       for (int64_t k = A.rowptr[i]; k < A.rowptr[i + 1]; ++k) {
         const int col = A.colind[k];
-        if (!HASB && col == i) continue;
+        if (FOLD && col == i) continue;
         scol[o] = col;
         if constexpr (ACPLX) sval[o] = csr_val(A, k); else sval[o] = A.val[k];
         ++o;
@@ -113,7 +117,7 @@ __global__ void __launch_bounds__(kMsThreads, 4)
               csr_fma<BCPLX>(bx, B, k, Xj[(size_t)B.colind[k] * m]);
             cfms(acc, zs[0][j], bx);
           } else {
-            cfms(acc, zs[r][j], Xj[(size_t)i * m]);
+            cfms(acc, zs[FOLD ? r : 0][j], Xj[(size_t)i * m]);
           }
           if (staged) {
             const int ke = send[r];
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(kMsThreads, 4)
           } else {
             for (int64_t k = A.rowptr[i]; k < A.rowptr[i + 1]; ++k) {
               const int col = A.colind[k];
-              if (HASB || col != i) csr_fma<ACPLX>(acc, A, k, Xj[(size_t)col * m]);
+              if (!FOLD || col != i) csr_fma<ACPLX>(acc, A, k, Xj[(size_t)col * m]);
             }
           }
           const cx<Tout> ro = ccast<Tout>(acc);
@@ -203,17 +207,19 @@ static int ms_grid(int n) {
   return g < 1 ? 1 : g;
 }
 
-#define MS_LAUNCH(AC, BC, HB, SKIP)                                                                         \
-  k_multishift_residual<Tout, AC, BC, HB><<<g, kMsThreads, 0, s>>>(A, Bv, ne, d_z, d_w, X, xns, BY, R, Q, \
-                                                                   partial, m, rpc, SKIP)
+#define MS_LAUNCH(AC, BC, HB, LG, SKIP)                                                                     \
+  k_multishift_residual<Tout, AC, BC, HB, LG><<<g, kMsThreads, 0, s>>>(A, Bv, ne, d_z, d_w, X, xns, BY, R, Q, \
+                                                                       partial, m, rpc, SKIP)
 #define MS_CALL(SKIP)                                                                                       \
   do {                                                                                                      \
-    if (!B) {                                                                                               \
-      if (A.cplx) MS_LAUNCH(true, false, false, SKIP); else MS_LAUNCH(false, false, false, SKIP);           \
+    if (!B && A.nnz > 128 * (int64_t)A.n) {                                                                 \
+      if (A.cplx) MS_LAUNCH(true, false, false, true, SKIP); else MS_LAUNCH(false, false, false, true, SKIP); \
+    } else if (!B) {                                                                                        \
+      if (A.cplx) MS_LAUNCH(true, false, false, false, SKIP); else MS_LAUNCH(false, false, false, false, SKIP); \
     } else if (A.cplx) {                                                                                    \
-      if (bc) MS_LAUNCH(true, true, true, SKIP); else MS_LAUNCH(true, false, true, SKIP);                   \
+      if (bc) MS_LAUNCH(true, true, true, false, SKIP); else MS_LAUNCH(true, false, true, false, SKIP);     \
     } else {                                                                                                \
-      if (bc) MS_LAUNCH(false, true, true, SKIP); else MS_LAUNCH(false, false, true, SKIP);                 \
+      if (bc) MS_LAUNCH(false, true, true, false, SKIP); else MS_LAUNCH(false, false, true, false, SKIP);   \
     }                                                                                                       \
   } while (0)
 
