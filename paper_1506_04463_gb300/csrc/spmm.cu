@@ -854,8 +854,12 @@ static void spmm_f32_launch(const CsrView &A, const CsrView *B, int bw, int long
 
 void launch_multishift_spmm_f32(const CsrView &A, const CsrView *B, int bw, int longest, int ne, const cxd *d_z,
                                 int conj_z, const cxf *P, cxf *V, int m, cudaStream_t s) {
-  // the fewest lanes a row that cover it in one pass
-  const int cols = ceil_div(m, 2);
+  // the fewest lanes a row that cover it in one pass; where long rows are too few
+  // to fill the chip, sixteen, which gather more of a row at once (us, 8 nodes,
+  // 600 rows of 600: 1 column 668 -> 447, 8 columns 793 -> 404; 3000 rows of 100, 8
+  // columns 152 -> 87; 6000 rows of 60 the other way, 103 -> 70 for 70 -> 111)
+  const bool few_long = A.nnz > 16 * (int64_t)A.n && A.n <= 3648;
+  const int cols = few_long ? std::max(9, ceil_div(m, 2)) : ceil_div(m, 2);
 #define SPG(PAIR)                                                                                     \
   do {                                                                                                \
     if (cols <= 4) return spmm_f32_launch<PAIR, 4>(A, B, bw, longest, ne, d_z, conj_z, P, V, m, s);   \

@@ -11,6 +11,7 @@ if not torch.cuda.is_available():
 
 from paper_1506_04463_gb300 import feast_nh as F  # noqa: E402
 from paper_1506_04463_gb300 import workloads as wl  # noqa: E402
+import test_gpu_spmm_groups  # noqa: E402
 from gpu_helpers import host  # noqa: E402
 
 
@@ -39,3 +40,12 @@ def test_rows(side, n, m, ne, per_row, span, cplx):
         ref, mag = zj * Pj - Ah @ Pj, abs(zj) * abs(Pj) + abs(Ah) @ abs(Pj)
         assert np.all(abs(V[j] - ref) <= 4 * (6 + per_row) * 2.0 ** -24 * mag)
     ctx.close()
+
+
+@pytest.mark.parametrize("side", [0, 1])
+@pytest.mark.parametrize("n,m,ne,per_row,cplx,withB", [
+    (300, 1, 2, 60, False, False), (301, 8, 3, 200, True, False), (300, 13, 2, 90, False, True), (3648, 7, 2, 18, False, False),
+    (3649, 7, 2, 18, False, False)])
+def test_few_long_rows(side, n, m, ne, per_row, cplx, withB):
+    """Sixteen lanes a row for few columns."""
+    test_gpu_spmm_groups.test_operator(side, n, m, ne, per_row, cplx, withB)
